@@ -17,54 +17,90 @@ static int gridn(int64_t n, int bs) {
   return (int)(g < 1 ? 1 : (g > 8192 ? 8192 : g));
 }
 
-// y[:, r] = A x[:, r]; one warp per row, lanes over the row's entries
-__global__ void k_spmv(int64_t N, const int64_t* rowptr, const int32_t* col, const double* val, const double* x,
-                       int64_t ldx, double* y, int64_t ldy, int nrhs) {
-  int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t row = w; row < N; row += nw) {
-    int64_t e0 = rowptr[row], e1 = rowptr[row + 1];
-    for (int r = 0; r < nrhs; ++r) {
-      double s = 0;
-      for (int64_t e = e0 + lane; e < e1; e += 32) s += val[e] * x[col[e] + r * ldx];
+// y[:, r] = A x[:, r], or b[:, r] - A x[:, r] when RES.  Eight lanes own a
+// row (edge elements: about 16 entries a row, two a lane) and carry up to R
+// columns in registers, so the matrix is read once per R columns and the R
+// gathers of an entry are in flight together.  The 8 partial sums of each
+// column meet by recursive halving: every step sends the columns the other
+// half of the lanes keeps, 7 exchanges for 8 columns, and lane c ends with
+// column c.  Bound by the gathers of x, which hit L1 and L2 (the edges of one
+// vertex are neighbours in the DOF order).
+template <int R>
+__device__ __forceinline__ double halve_columns(double (&acc)[R], int lane) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) y[row + r * ldy] = s;
+  for (int w = R, o = 4; o > 0; o >>= 1) {
+    if (w > 1) {
+      w >>= 1;
+      const bool hi = (lane & o) != 0;
+#pragma unroll
+      for (int q = 0; q < R / 2; ++q)
+        if (q < w) {
+          const double keep = hi ? acc[q + w] : acc[q], send = hi ? acc[q] : acc[q + w];
+          acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    } else {
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+    }
+  }
+  return acc[0];
+}
+template <int R, bool RES>
+__global__ void __launch_bounds__(256) k_spmv(int64_t N, const int64_t* __restrict__ rowptr,
+                                              const int32_t* __restrict__ col, const double* __restrict__ val,
+                                              const double* __restrict__ x, int64_t ldx, const double* b, int64_t ldb,
+                                              double* y, int64_t ldy, int nrhs) {
+  const int lane = threadIdx.x & 7;
+  const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) >> 3;
+  // whole warps stay in the loop together (the exchanges are warp-wide)
+  const int64_t first = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
+  for (int64_t row = first; row - ((threadIdx.x & 31) >> 3) < N; row += ngrp) {
+    const bool in = row < N;
+    const int64_t e0 = in ? rowptr[row] : 0, e1 = in ? rowptr[row + 1] : 0;
+    for (int r0 = 0; r0 < nrhs; r0 += R) {
+      const int nr = nrhs - r0;
+      const double* xr = x + (int64_t)r0 * ldx;
+      double acc[R];
+#pragma unroll
+      for (int q = 0; q < R; ++q) acc[q] = 0.0;
+#pragma unroll 2
+      for (int64_t e = e0 + lane; e < e1; e += 8) {
+        const double v = val[e];
+        const double* xc = xr + col[e];
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+          if (q < nr) acc[q] += v * xc[q * ldx];
+      }
+      const double s = halve_columns<R>(acc, lane);
+      // lane bits 4, 2, 1 chose halves of 4, 2, 1 columns
+      const int c = R == 8 ? lane : 0;
+      if (in && (R == 8 ? c < nr : lane == 0)) {
+        const int64_t o = row + (int64_t)(r0 + c) * ldy;
+        y[o] = RES ? b[row + (int64_t)(r0 + c) * ldb] - s : s;
+      }
     }
   }
 }
-
+// One column: R = 1.  More: R = 8, the last group guarded (n = 24: 8 columns
+// 45 us, the warp-per-row kernel before it, one column at a time, 270 us).
+template <bool RES>
+static void launch_spmv(const int64_t* rowptr, const int32_t* col, const double* val, int64_t N, const double* x,
+                        int64_t ldx, const double* b, int64_t ldb, double* y, int64_t ldy, int nrhs, cudaStream_t s) {
+  note_launch();
+  const int g = gridn(N * 8, 256);
+  if (nrhs == 1)
+    k_spmv<1, RES><<<g, 256, 0, s>>>(N, rowptr, col, val, x, ldx, b, ldb, y, ldy, nrhs);
+  else
+    k_spmv<8, RES><<<g, 256, 0, s>>>(N, rowptr, col, val, x, ldx, b, ldb, y, ldy, nrhs);
+}
 cudaError_t spmv(const int64_t* rowptr, const int32_t* col, const double* val, int64_t N, const double* x,
                  int64_t ldx, double* y, int64_t ldy, int nrhs, cudaStream_t s) {
-  int64_t threads = N * 32;
-  note_launch();
-  k_spmv<<<gridn(threads, 256), 256, 0, s>>>(N, rowptr, col, val, x, ldx, y, ldy, nrhs);
+  launch_spmv<false>(rowptr, col, val, N, x, ldx, nullptr, 0, y, ldy, nrhs, s);
   return cudaGetLastError();
 }
-
 // out = b - A x
-__global__ void k_residual(int64_t N, const int64_t* rowptr, const int32_t* col, const double* val, const double* x,
-                           int64_t ldx, const double* b, int64_t ldb, double* out, int64_t ldo, int nrhs) {
-  int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t row = w; row < N; row += nw) {
-    int64_t e0 = rowptr[row], e1 = rowptr[row + 1];
-    for (int r = 0; r < nrhs; ++r) {
-      double s = 0;
-      for (int64_t e = e0 + lane; e < e1; e += 32) s += val[e] * x[col[e] + r * ldx];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) out[row + r * ldo] = b[row + r * ldb] - s;
-    }
-  }
-}
-
 cudaError_t residual(const int64_t* rowptr, const int32_t* col, const double* val, int64_t N, const double* x,
                      int64_t ldx, const double* b, int64_t ldb, double* out, int64_t ldo, int nrhs, cudaStream_t s) {
-  note_launch();
-  k_residual<<<gridn(N * 32, 256), 256, 0, s>>>(N, rowptr, col, val, x, ldx, b, ldb, out, ldo, nrhs);
+  launch_spmv<true>(rowptr, col, val, N, x, ldx, b, ldb, out, ldo, nrhs, s);
   return cudaGetLastError();
 }
 
