@@ -277,7 +277,7 @@ int hlu_factor_stats(const hlu_handle* h, hlu_factor_info* info);
  * out[3*k + 0] tasks run, out[3*k + 1] SM clock cycles spent waiting for a
  * ready task, out[3*k + 2] cycles spent running, summed over CTAs; kinds
  * k = 0..8 are GETRF, TRSM_L, TRSM_UT, TRSM_U, PROJ, ROWMV, TRUNC, DADD,
- * RSOLVE and k = 9 the no-work fences; then the truncation phases summed
+ * (unused) and k = 9 the no-work fences; then the truncation phases summed
  * over all compressions: out[30] stacking (shared-memory route) or dense
  * sum, out[31] QR cycles, out[32] core product, out[33] Jacobi SVD, out[34]
  * selection and Q application, out[35] compressions, out[36] Jacobi sweeps,

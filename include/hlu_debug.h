@@ -166,6 +166,11 @@ int hlu_debug_host_hinverse(int32_t nc, const int32_t* clusters, int32_t nb, con
  * Returns HLU_ERR_TIMEOUT when the wait ran out as intended. */
 int hlu_debug_wait_timeout(double limit_ms, int32_t* status_out);
 
+/* hlu_debug_solve_wait_timeout - the same for the triangular solve's launch:
+ * its only task waits for itself, so the bounded wait runs out after limit_ms
+ * and the call returns HLU_ERR_TIMEOUT with status_out as above. */
+int hlu_debug_solve_wait_timeout(double limit_ms, int32_t* status_out);
+
 #ifdef __cplusplus
 }
 #endif

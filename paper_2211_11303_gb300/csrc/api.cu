@@ -132,10 +132,13 @@ struct DevSched {
     if ((e = upload(&roots, rq)) != cudaSuccess) return e;
     return cudaSuccess;
   }
-  cudaError_t alloc_state() {
+  // with_queue: false for the triangular solve, whose tasks are handed out by
+  // tickets (qctl[0])
+  cudaError_t alloc_state(bool with_queue = true) {
     cudaError_t e = dev_malloc(&indeg, sizeof(int32_t) * std::max<int64_t>(ntasks, 1));
     if (e != cudaSuccess) return e;
-    if ((e = dev_malloc(&queue, sizeof(unsigned long long) * std::max<int64_t>(ntasks, 1))) != cudaSuccess) return e;
+    if (with_queue && (e = dev_malloc(&queue, sizeof(unsigned long long) * std::max<int64_t>(ntasks, 1))) != cudaSuccess)
+      return e;
     return dev_malloc(&qctl, sizeof(unsigned long long) * 2);
   }
   // a per-handle view of shared task data
@@ -177,10 +180,14 @@ struct SchedBundle {
   FillDesc* d_fill_lr = nullptr;
   int32_t n_fill_dense = 0, n_fill_lr = 0;
   int64_t dense_rows = 0;
+  InvUnit* d_inv_units = nullptr;    // the solve blocks' inverses (L.inv_units, L.inv_leaves)
+  InvLeaf* d_inv_leaves = nullptr;
   int64_t device_bytes = 0;  // task data of both schedules on the device
   ~SchedBundle() {
     dF.free_all();
     dS.free_all();
+    if (d_inv_units) dev_free(d_inv_units);
+    if (d_inv_leaves) dev_free(d_inv_leaves);
     if (d_fill_dense) dev_free(d_fill_dense);
     if (d_fill_lr) dev_free(d_fill_lr);
   }
@@ -326,10 +333,9 @@ namespace {
 void free_factor(hlu_handle* h) {
   for (void* p : {(void*)h->d_arena, (void*)h->d_ranks, (void*)h->d_piv, (void*)h->d_scratch, (void*)h->d_status,
                   (void*)h->d_flops, (void*)h->d_arenas, (void*)h->d_rankp, (void*)h->d_pivp,
-                  (void*)h->d_prof, (void*)h->d_term_p})
+                  (void*)h->d_prof})
     if (p) dev_free(p);
   h->d_prof = nullptr;
-  h->d_term_p = nullptr;
   h->term_p_fresh = false;
   h->d_arena = nullptr;
   h->d_ranks = nullptr;
@@ -364,20 +370,49 @@ __global__ void k_term_ranks(const Term* terms, int64_t n, const int32_t* ranks,
   }
 }
 
-// Before a launch of schedule ds on h: a factorisation makes the resolved
-// term widths stale; a solve launch refreshes them (stream-ordered after the
-// factorisation that produced the ranks).
-int prepare_terms(hlu_handle* h, DevSched& ds, cudaStream_t s) {
-  if (&ds == &h->dF) {
-    h->term_p_fresh = false;
-    return HLU_OK;
-  }
-  if (&ds != &h->dS || ds.nterms == 0 || !h->d_term_p || h->term_p_fresh) return HLU_OK;
-  const int blocks = (int)std::min<int64_t>((ds.nterms + 255) / 256, 1184);
+// The term widths of h's triangular solve, resolved before the first solve
+// after a factorisation (stream-ordered after the ranks it produced).
+int prepare_terms(hlu_handle* h, cudaStream_t s) {
+  if (h->dS.nterms == 0 || h->term_p_fresh) return HLU_OK;
+  const int blocks = (int)std::min<int64_t>((h->dS.nterms + 255) / 256, 1184);
   note_launch();
-  k_term_ranks<<<blocks, 256, 0, s>>>(ds.terms, ds.nterms, h->d_ranks, h->L.nrhs_slot, h->d_term_p);
+  k_term_ranks<<<blocks, 256, 0, s>>>(h->dS.terms, h->dS.nterms, h->d_ranks, h->L.nrhs_slot, h->d_term_p);
   CKR(cudaGetLastError(), "term widths");
   h->term_p_fresh = true;
+  return HLU_OK;
+}
+
+// One launch of the triangular solves of several handles with the same
+// precision, on the columns in their work vectors.  Handle 0's status is used.
+int solve_run(hlu_handle* const* hs, int count, cudaStream_t s) {
+  if (count < 1 || count > kMaxBatch) return fail(HLU_ERR_ARG, "batch size");
+  SolveArgs a;
+  std::memset(&a, 0, sizeof(a));
+  for (int i = 0; i < count; ++i) {
+    hlu_handle* h = hs[i];
+    if (h->precision != hs[0]->precision) return fail(HLU_ERR_ARG, "mixed precisions in a batch");
+    for (int j = 0; j < i; ++j)
+      if (hs[j] == h) return fail(HLU_ERR_ARG, "a handle appears twice in a batch");
+    if (int rc = prepare_terms(h, s)) return rc;
+    SolveProb& p = a.probs[i];
+    p.tasks = h->dS.tasks;
+    p.terms = h->dS.terms;
+    p.term_p = h->d_term_p;
+    p.succ_ptr = h->dS.succ_ptr;
+    p.succ_idx = h->dS.succ_idx;
+    p.indeg0 = h->dS.indeg0;
+    p.indeg = h->dS.indeg;
+    p.ticket = h->dS.qctl;
+    p.arena = h->d_arena;
+    p.ranks = h->d_ranks;
+    p.ntasks = h->dS.ntasks;
+    p.nrhs = h->cur_nrhs;
+  }
+  a.nprobs = count;
+  a.status = hs[0]->d_status;
+  a.wait_limit_ns = (unsigned long long)(g_wait_limit_ms * 1e6);
+  a.trace = count == 1 ? hs[0]->d_trace : nullptr;
+  CKR(hs[0]->precision == HLU_FP64 ? solve_launch<double>(a, s) : solve_launch<float>(a, s), "solve launch");
   return HLU_OK;
 }
 
@@ -398,7 +433,6 @@ ProbSched prob_of(hlu_handle* h, DevSched& ds, int64_t limit) {
   p.limit = ds.run_count(limit);
   p.nrhs_slot = h->L.nrhs_slot;
   p.nrhs = h->cur_nrhs;
-  p.term_p = (&ds == &h->dS && h->term_p_fresh) ? h->d_term_p : nullptr;
   return p;
 }
 
@@ -435,7 +469,6 @@ cudaError_t launch_exec(int precision, const ExecArgs& a, int g, cudaStream_t s)
 // One launch of the executor over one problem's schedule (or its first
 // `limit` tasks): counters reset, queue cleared and seeded with the roots.
 int exec_run(hlu_handle* h, DevSched& ds, int grid, cudaStream_t s, bool with_flops, int64_t limit = -1) {
-  if (int rc = prepare_terms(h, ds, s)) return rc;
   ExecArgs a;
   std::memset(&a, 0, sizeof(a));
   a.probs[0] = prob_of(h, ds, limit);
@@ -484,12 +517,11 @@ std::vector<unsigned long long> batch_roots(const std::vector<const std::vector<
   return out;
 }
 
-// One launch over the factor (which = 0) or solve (which = 1) schedules of
-// several handles with the same precision.  Handle 0's status, flop counter
-// and profile are used; the scratch is that of the handle with the largest
-// truncation stacks; the queue (all problems' tasks) lives in *d_q.
-int exec_run_batch(hlu_handle* const* hs, int count, int which, cudaStream_t s, unsigned long long** d_q,
-                   int64_t* d_q_len) {
+// One launch over the factor schedules of several handles with the same
+// precision.  Handle 0's status, flop counter and profile are used; the
+// scratch is that of the handle with the largest truncation stacks; the queue
+// (all problems' tasks) lives in *d_q.
+int exec_run_batch(hlu_handle* const* hs, int count, cudaStream_t s, unsigned long long** d_q, int64_t* d_q_len) {
   if (count < 1 || count > kMaxBatch) return fail(HLU_ERR_ARG, "batch size");
   ExecArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -502,8 +534,7 @@ int exec_run_batch(hlu_handle* const* hs, int count, int which, cudaStream_t s, 
     if (h->precision != hs0->precision) return fail(HLU_ERR_ARG, "mixed precisions in a batch");
     for (int j = 0; j < i; ++j)
       if (hs[j] == h) return fail(HLU_ERR_ARG, "a handle appears twice in a batch");
-    DevSched& ds = which == 0 ? h->dF : h->dS;
-    if (int rc = prepare_terms(h, ds, s)) return rc;
+    DevSched& ds = h->dF;
     a.probs[i] = prob_of(h, ds, -1);
     roots[i] = &ds.h_roots;
     total += ds.ntasks;
@@ -522,13 +553,13 @@ int exec_run_batch(hlu_handle* const* hs, int count, int which, cudaStream_t s, 
   }
   a.qctl = *d_q;
   a.queue = *d_q + 2;
-  fill_common(a, big, hs0, which == 0);
+  fill_common(a, big, hs0, true);
   int32_t st0[8] = {0, -1, 0, 0, 0, 0, 0, 0};
   unsigned long long q0[2] = {0ULL, (unsigned long long)seed.size()};
   CKR(cudaMemcpyAsync(hs0->d_status, st0, sizeof(st0), cudaMemcpyHostToDevice, s), "status reset");
   CKR(cudaMemcpyAsync(a.qctl, q0, sizeof(q0), cudaMemcpyHostToDevice, s), "queue reset");
   for (int i = 0; i < count; ++i) {
-    DevSched& ds = which == 0 ? hs[i]->dF : hs[i]->dS;
+    DevSched& ds = hs[i]->dF;
     CKR(cudaMemcpyAsync(ds.indeg, ds.indeg0, sizeof(int32_t) * ds.ntasks, cudaMemcpyDeviceToDevice, s), "counters");
   }
   CKR(cudaMemcpyAsync(a.queue, seed.data(), sizeof(unsigned long long) * seed.size(), cudaMemcpyHostToDevice, s),
@@ -562,7 +593,7 @@ int solve_impl(const hlu_handle* hc, const double* b, double* x, int32_t nrhs, i
     CKR(set_int(h->d_ranks + h->L.nrhs_slot, nc, s), "nrhs slot");
     h->cur_nrhs = nc;
     CKR(gather_cast<T>(N, h->d_perm, b + c0 * ld, ld, work, nc, s), "gather");
-    int rc = exec_run(h, h->dS, h->grid, s, false);
+    int rc = solve_run(&h, 1, s);
     if (rc) return rc;
     CKR(scatter_cast<T>(N, h->d_perm, work, x + c0 * ld, ld, nc, s), "scatter");
   }
@@ -591,7 +622,6 @@ int exec_run_inv(hlu_handle* h, DevSched& ds, double alpha, int32_t nrhs, cudaSt
   p.limit = ds.ntasks;
   p.nrhs_slot = iv.L.nrhs_slot;
   p.nrhs = nrhs;
-  p.term_p = nullptr;
   p.alpha = alpha;
   a.nprobs = 1;
   a.ntotal = ds.ntasks;
@@ -891,7 +921,7 @@ void hlu_destroy(hlu_handle* h) {
   for (void* p : {(void*)h->mesh.dofmap, (void*)h->mesh.edges, (void*)h->mesh.pts, (void*)h->mesh.xyz,
                   (void*)h->mesh.tets, (void*)h->mesh.ekeys, (void*)h->mesh.beta, (void*)h->A.rowptr,
                   (void*)h->A.col, (void*)h->A.val,
-                  (void*)h->d_perm, (void*)h->d_iperm})
+                  (void*)h->d_perm, (void*)h->d_iperm, (void*)h->d_term_p})
     if (p) dev_free(p);
   if (h->ev0) cudaEventDestroy(h->ev0);
   if (h->ev1) cudaEventDestroy(h->ev1);
@@ -1027,6 +1057,8 @@ int hlu_build(const hlu_mesh* mesh, double kappa, int32_t leaf, double eta, doub
       sb->dense_rows = rows;
       if ((e = upload(&sb->d_fill_dense, fd)) != cudaSuccess) return bail(e, "fill desc");
       if ((e = upload(&sb->d_fill_lr, fl)) != cudaSuccess) return bail(e, "fill desc");
+      if ((e = upload(&sb->d_inv_units, sb->L.inv_units)) != cudaSuccess) return bail(e, "solve blocks");
+      if ((e = upload(&sb->d_inv_leaves, sb->L.inv_leaves)) != cudaSuccess) return bail(e, "solve blocks");
       for (const Schedule* sc : {&F, &S})
         sb->device_bytes += (int64_t)(sizeof(Task) * sc->tasks.size() +
                                       sizeof(Term) * sc->terms.size() + sizeof(Piece) * sc->pieces.size() +
@@ -1049,7 +1081,7 @@ int hlu_build(const hlu_mesh* mesh, double kappa, int32_t leaf, double eta, doub
     h->dF = h->sb->dF.share();
     h->dS = h->sb->dS.share();
     if ((e = h->dF.alloc_state()) != cudaSuccess) return bail(e, "queue");
-    if ((e = h->dS.alloc_state()) != cudaSuccess) return bail(e, "queue");
+    if ((e = h->dS.alloc_state(false)) != cudaSuccess) return bail(e, "tickets");
     if (h->dS.nterms > 0 && (e = dev_malloc(&h->d_term_p, sizeof(int32_t) * h->dS.nterms)) != cudaSuccess)
       return bail(e, "term widths");
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return bail(e, "sync");
@@ -1161,6 +1193,7 @@ static int factor_prepare(hlu_handle* h, int32_t precision, cudaStream_t s) {
     CKR(dev_malloc(&h->d_prof, sizeof(unsigned long long) * kProfEntries), "prof");
   }
   h->precision = precision;
+  h->term_p_fresh = false;
   CKR(cudaMemsetAsync(h->d_ranks, 0, sizeof(int32_t) * std::max(h->L.n_slots, 1), s), "ranks");
   h->cur_nrhs = 0;
   int32_t st0[8] = {0, -1, 0, 0, 0, 0, 0, 0};
@@ -1180,6 +1213,19 @@ static int factor_prepare(hlu_handle* h, int32_t precision, cudaStream_t s) {
   if (rc) return rc;
   CKR(cudaMemsetAsync(h->d_flops, 0, sizeof(double), s), "flops");
   CKR(cudaMemsetAsync(h->d_prof, 0, sizeof(unsigned long long) * kProfEntries, s), "prof");
+  return HLU_OK;
+}
+
+// after a factorisation was launched: the solve blocks' inverses
+static int factor_inverses(hlu_handle* h, cudaStream_t s) {
+  const SchedBundle& b = *h->sb;
+  const int32_t nu = (int32_t)b.L.inv_units.size(), nl = (int32_t)b.L.inv_leaves.size();
+  if (h->precision == HLU_FP64)
+    CKR(invert_blocks<double>(b.d_inv_units, nu, b.d_inv_leaves, nl, (double*)h->d_arena, h->d_ranks, h->d_piv, s),
+        "solve blocks");
+  else
+    CKR(invert_blocks<float>(b.d_inv_units, nu, b.d_inv_leaves, nl, (float*)h->d_arena, h->d_ranks, h->d_piv, s),
+        "solve blocks");
   return HLU_OK;
 }
 
@@ -1233,6 +1279,7 @@ static int factor_impl(hlu_handle* h, int32_t precision, void* stream, int64_t l
     CKR(cudaEventRecord(h->ev0, s), "event");
     rc = exec_run(h, h->dF, h->grid, s, true, limit);
     if (rc) return rc;
+    if (limit < 0 && (rc = factor_inverses(h, s))) return rc;
     CKR(cudaEventRecord(h->ev1, s), "event");
     CKR(cudaEventSynchronize(h->ev1), "sync");
     float ms = 0;
@@ -1257,6 +1304,7 @@ int hlu_factor_async(hlu_handle* h, int32_t precision, int32_t max_ctas, void* s
     const int grid = max_ctas > 0 ? std::min(h->grid, (int)max_ctas) : h->grid;
     rc = exec_run(h, h->dF, grid, s, true);
     if (rc) return rc;
+    if ((rc = factor_inverses(h, s))) return rc;
     CKR(cudaEventRecord(h->ev1, s), "event");
     h->factor_pending = true;
     h->factor_stream = s;
@@ -1644,8 +1692,10 @@ int hlu_factor_batch(hlu_handle** hs, int32_t count, int32_t precision, void* st
     }
     std::lock_guard<std::mutex> lk(g_batch_mu);
     CKR(cudaEventRecord(hs[0]->ev0, s), "event");
-    int rc = exec_run_batch(hs, count, 0, s, &g_batch_q, &g_batch_q_len);
+    int rc = exec_run_batch(hs, count, s, &g_batch_q, &g_batch_q_len);
     if (rc) return rc;
+    for (int32_t i = 0; i < count; ++i)
+      if ((rc = factor_inverses(hs[i], s))) return rc;
     CKR(cudaEventRecord(hs[0]->ev1, s), "event");
     CKR(cudaEventSynchronize(hs[0]->ev1), "sync");
     float ms = 0;
@@ -1685,11 +1735,7 @@ int hlu_solve_batch(hlu_handle* const* hs, int32_t count, const double* const* b
         CKR(gather_cast<float>(h->A.N, h->d_perm, b[i], h->A.N, (float*)h->d_arena + h->L.work_off, nrhs[i], s),
             "gather");
     }
-    {
-      std::lock_guard<std::mutex> lk(g_batch_mu);
-      int rc = exec_run_batch(hs, count, 1, s, &g_batch_q, &g_batch_q_len);
-      if (rc) return rc;
-    }
+    if (int rc = solve_run(hs, count, s)) return rc;
     for (int32_t i = 0; i < count; ++i) {
       hlu_handle* h = hs[i];
       if (h->precision == HLU_FP64)
@@ -1767,6 +1813,49 @@ extern "C" int hlu_debug_wait_timeout(double limit_ms, int32_t* status_out) {
   return rc;
 }
 
+// The same for the triangular solve's launch: the one task waits for itself.
+extern "C" int hlu_debug_solve_wait_timeout(double limit_ms, int32_t* status_out) {
+  if (!status_out || !(limit_ms > 0) || limit_ms > 5000) return fail(HLU_ERR_ARG, "bad argument");
+  Schedule S;
+  Task t;
+  std::memset(&t, 0, sizeof(t));
+  t.type = TK_NUM;  // no work
+  t.out_slot = -1;
+  S.tasks = {t};
+  S.pred_ptr = {0, 1};
+  S.pred_idx = {0};
+  DevSched ds;
+  int32_t* d_status = nullptr;
+  cudaError_t e = ds.load(S);
+  if (e == cudaSuccess) e = ds.alloc_state(false);
+  if (e == cudaSuccess) e = dev_malloc(&d_status, sizeof(int32_t) * 8);
+  int32_t st[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  if (e == cudaSuccess) {
+    SolveArgs a;
+    std::memset(&a, 0, sizeof(a));
+    SolveProb& p = a.probs[0];
+    p.tasks = ds.tasks;
+    p.succ_ptr = ds.succ_ptr;
+    p.succ_idx = ds.succ_idx;
+    p.indeg0 = ds.indeg0;
+    p.indeg = ds.indeg;
+    p.ticket = ds.qctl;
+    p.ntasks = ds.ntasks;
+    p.nrhs = 1;
+    a.nprobs = 1;
+    a.status = d_status;
+    a.wait_limit_ns = (unsigned long long)(limit_ms * 1e6);
+    e = solve_launch<float>(a, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpy(st, d_status, sizeof(st), cudaMemcpyDeviceToHost);
+  }
+  ds.free_all();
+  if (d_status) dev_free(d_status);
+  CKR(e, "solve wait test");
+  status_out[0] = st[0];
+  status_out[1] = st[1];
+  return st[0] == 5 ? fail(HLU_ERR_TIMEOUT, "device wait exceeded its limit") : HLU_OK;
+}
+
 // Runs A_H fill and the first `limit` tasks of the factorisation DAG, then
 // copies the arena (elements, in the factor precision) and the rank slots to
 // host buffers; sizes[0] = arena elements, sizes[1] = rank slots, sizes[2] =
@@ -1836,7 +1925,7 @@ extern "C" int hlu_debug_solve_trace(hlu_handle* h, int32_t nrhs, uint64_t* trac
   CKR(cudaMemset(h->d_trace, 0, sizeof(unsigned long long) * 4 * std::max<int64_t>(nt, 1)), "trace");
   CKR(set_int(h->d_ranks + h->L.nrhs_slot, nrhs, nullptr), "nrhs slot");
   h->cur_nrhs = nrhs;
-  int rc = exec_run(h, h->dS, h->grid, nullptr, false);
+  int rc = solve_run(&h, 1, nullptr);
   if (!rc) {
     int32_t st[8];
     rc = read_status(h, nullptr, st);
@@ -2120,11 +2209,7 @@ int solve_segments(std::vector<hlu_handle*>& hs, std::vector<std::vector<SolveSe
     CKR(set_int(h->d_ranks + h->L.nrhs_slot, off, s), "nrhs slot");
     h->cur_nrhs = off;
   }
-  {
-    std::lock_guard<std::mutex> lk(g_batch_mu);
-    int rc = exec_run_batch(hs.data(), (int)hs.size(), 1, s, &g_batch_q, &g_batch_q_len);
-    if (rc) return rc;
-  }
+  if (int rc = solve_run(hs.data(), (int)hs.size(), s)) return rc;
   for (size_t i = 0; i < hs.size(); ++i) {
     hlu_handle* h = hs[i];
     int off = 0;

@@ -136,6 +136,7 @@ extern "C" int hlu_debug_host_factor_prefix(int32_t nc, const int32_t* clusters,
         if (ranks_out) std::memcpy(ranks_out, ranks.data(), sizeof(int32_t) * ranks.size());
         return st1;
       }
+      host_invert<float>(L, af.data(), ranks.data(), piv.data());
       ranks[L.nrhs_slot] = nrhs;
       for (int32_t j = 0; j < nrhs; ++j)
         for (int32_t i = 0; i < N; ++i) af[L.work_off + i + (int64_t)j * N] = (float)b[perm[i] + (int64_t)j * N];
@@ -149,6 +150,7 @@ extern "C" int hlu_debug_host_factor_prefix(int32_t nc, const int32_t* clusters,
         if (ranks_out) std::memcpy(ranks_out, ranks.data(), sizeof(int32_t) * ranks.size());
         return st1;
       }
+      host_invert<double>(L, arena.data(), ranks.data(), piv.data());
       // solve: work vector in permuted order
       ranks[L.nrhs_slot] = nrhs;
       for (int32_t j = 0; j < nrhs; ++j)

@@ -98,7 +98,6 @@ struct Ctx {
   double jacobi_tol;
   int32_t compress_at;
   int32_t nrhs_slot, nrhs;  // the launch's right-hand-side count and its slot
-  const int32_t* term_p;    // resolved term column counts (solve launches) or null
   TcCtl* tcc;               // tensor-core tile products (FP32 factorisations with TF32) or null
   double alpha;             // the launch's scalar for TF_ALPHA / PF_ALPHA
 };
@@ -691,10 +690,8 @@ __device__ double rowmv_tile(const Ctx<T>& c, const Task& t, int i0, int j0, int
       int32_t* dst = reinterpret_cast<int32_t*>(s_tm);
       for (int w = threadIdx.x; w < words; w += NT) dst[w] = __ldg(src + w);
     }
-    // resolved column counts arrive with the terms (no dependent rank load)
-    const int pq = (c.term_p && threadIdx.x < nq) ? __ldcg(c.term_p + t.list_begin + qb + threadIdx.x) : -1;
     __syncthreads();
-    if (threadIdx.x < nq) s_p[threadIdx.x] = pq >= 0 ? pq : ncols(c, s_tm[threadIdx.x].A);
+    if (threadIdx.x < nq) s_p[threadIdx.x] = ncols(c, s_tm[threadIdx.x].A);
     __syncthreads();
     TermCursor<T> cur{&c, s_tm, s_p, nq, i0, j0, k, 0, 0};
     tile_mma_seq(acc, cur, As, Bs, c.tcc);
@@ -708,7 +705,13 @@ __device__ double rowmv_tile(const Ctx<T>& c, const Task& t, int i0, int j0, int
 }
 
 template <class T>
-__device__ __forceinline__ void cp_async_elem(T* sdst, const T* gsrc);
+__device__ __forceinline__ void cp_async_elem(T* sdst, const T* gsrc) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(sdst);
+  if (sizeof(T) == 4)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(gsrc) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"(gsrc) : "memory");
+}
 
 template <class T>
 __device__ void task_rowmv(Ctx<T>& c, const Task& t, char* smem) {
@@ -758,109 +761,6 @@ __device__ void task_rowmv(Ctx<T>& c, const Task& t, char* smem) {
     c.flops += fl;
     if (t.out_slot >= 0) __stcg(c.ranks + t.out_slot, k);
   }
-}
-
-// ---------------------------------------------------------------- RSOLVE
-// A leaf of a triangular solve with its late update: c -= sum_t A_t B_t, then
-// the diagonal tile's triangle (L^-1 P or U^-1) in place.  The tile streams
-// into shared memory (cp.async) while the update runs, and the updated
-// right-hand side goes to the substitution through shared memory.
-template <class T>
-__device__ __forceinline__ void cp_async_elem(T* sdst, const T* gsrc) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(sdst);
-  if (sizeof(T) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(gsrc) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"(gsrc) : "memory");
-}
-
-template <class T>
-__device__ void task_rsolve(Ctx<T>& c, const Task& t, char* smem) {
-  const int n = t.a.rows, k = ncols(c, t.b);
-  const bool upper = (t.flags & TF_UPPER) != 0;
-  if (n > 64 || k > 64) {  // not a leaf tile: update, then the plain leaf solve
-    Task r = t;
-    r.type = TK_ROWMV;
-    r.flags = 0;
-    r.out_slot = -1;
-    task_rowmv(c, r, smem);
-    __threadfence_block();
-    __syncthreads();
-    Task q = t;
-    q.type = upper ? TK_TRSM_U : TK_TRSM_L;
-    q.b = t.c;
-    task_trsm(c, q, smem);
-    return;
-  }
-  T* As = reinterpret_cast<T*>(smem);
-  T* Bs = As + kStage;
-  T* A = Bs + kStage;  // the diagonal tile, n x n
-  T* X = A + 64 * 64;   // updated right-hand side, n x k (ld n)
-  T* dinv = X + 64 * 64;
-  int* perm = reinterpret_cast<int*>(dinv + 64);
-  // the tile and the right-hand side start moving now: the tile is read-only
-  // factor data, and no other task touches this segment of the right-hand
-  // side while this one runs.  All the view's columns are copied (the work
-  // vector holds that many), so the copy need not wait for the live count.
-  const T* tile = c.arena + t.a.off;
-  for (int idx = threadIdx.x; idx < n * n; idx += NT)
-    cp_async_elem(A + idx, tile + (int64_t)(idx % n) * t.a.rs + (int64_t)(idx / n) * t.a.cs);
-  const int kx = min(t.c.cols, 64);
-  const T* rhs = c.arena + t.c.off;
-  for (int idx = threadIdx.x; idx < n * kx; idx += NT)
-    cp_async_elem(X + idx, rhs + (int64_t)(idx % n) * t.c.rs + (int64_t)(idx / n) * t.c.cs);
-  asm volatile("cp.async.commit_group;" ::: "memory");
-  const int pv = (!upper && threadIdx.x < n) ? __ldcg(c.piv + t.piv_off + threadIdx.x) : 0;
-  // the update, kept in registers
-  T acc[4][4];
-  acc_zero(acc);
-  double fl = t.list_count > 0 ? rowmv_tile(c, t, 0, 0, k, acc, As, Bs) : 0.0;
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncthreads();
-  if (t.list_count > 0) {
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const T sg = T(t.sign);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int r = tx * 4 + i, cc = ty * 4 + j;
-        if (r < n && cc < k) X[r + cc * n] += sg * acc[i][j];
-      }
-  }
-  if (!upper && threadIdx.x < n) perm[threadIdx.x] = pv;
-  __syncthreads();
-  if (upper)
-    for (int i = threadIdx.x; i < n; i += NT) dinv[i] = T(1) / A[i + i * n];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = lane, r1 = lane + 32;
-  for (int j = warp; j < k; j += NT / 32) {
-    const T* xj = X + j * n;
-    T v0 = 0, v1 = 0;
-    if (!upper) {
-      if (r0 < n) v0 = xj[perm[r0]];
-      if (r1 < n) v1 = xj[perm[r1]];
-      for (int l = 0; l < n; ++l) {
-        T x = __shfl_sync(0xffffffffu, l < 32 ? v0 : v1, l & 31);
-        if (r0 > l && r0 < n) v0 -= A[r0 + l * n] * x;
-        if (r1 > l && r1 < n) v1 -= A[r1 + l * n] * x;
-      }
-    } else {
-      if (r0 < n) v0 = xj[r0];
-      if (r1 < n) v1 = xj[r1];
-      for (int l = n - 1; l >= 0; --l) {
-        T x = __shfl_sync(0xffffffffu, l < 32 ? v0 : v1, l & 31) * dinv[l];
-        if (r0 == l) v0 = x;
-        if (r1 == l) v1 = x;
-        if (r0 < l) v0 -= A[r0 + l * n] * x;
-        if (r1 < l && r1 < n) v1 -= A[r1 + l * n] * x;
-      }
-    }
-    if (r0 < n) stv(c, t.c, r0, j, v0);
-    if (r1 < n) stv(c, t.c, r1, j, v1);
-  }
-  if (threadIdx.x == 0) c.flops += fl + (double)n * n * k;
 }
 
 // ---------------------------------------------------------------- DADD
@@ -1214,8 +1114,8 @@ constexpr int kCoreRank = kRankMax;      // rows kept by the stack route's pivot
 constexpr int kCoreV = kTruncStack * kCoreRank + kCoreRank * kCoreRank;  // M (q x r') and V (r' x r')
 
 // dynamic shared memory of the task bodies: max over task kinds of TRUNC
-// (3 stack-wide vectors + G + V), GETRF/TRSM (64 x 64 + 64 ints), the fused
-// leaf solve and the staged GEMM chunks (2 x KC x kLds)
+// (3 stack-wide vectors + G + V), GETRF/TRSM (64 x 64 + 64 ints) and the staged
+// GEMM chunks (2 x KC x kLds) with a ROWMV's output tile
 __host__ __device__ constexpr size_t exec_smem_base(int elem_size) {
   const size_t trunc0 = (size_t)elem_size * (3 * kTruncStack + kTruncStack * kTruncStack + kCoreV);
   // dense truncation route (FP32 only)
@@ -1224,11 +1124,8 @@ __host__ __device__ constexpr size_t exec_smem_base(int elem_size) {
   const size_t dense = region0 + (size_t)4 * (kDenseMax * kDenseMax + 2 * kDenseMax) + sizeof(int) * kDenseMax;
   const size_t trunc = (elem_size == 4 && dense > trunc0) ? dense : trunc0;
   const size_t lu0 = (size_t)elem_size * (64 * 64 + 64) + 64 * sizeof(int);
-  // fused leaf solve: staging chunks, tile, right-hand side, inverse diagonal, pivots
-  const size_t rsolve = (size_t)elem_size * (2 * kStage + 2 * 64 * 64 + 64) + 64 * sizeof(int);
-  const size_t lu = rsolve > lu0 ? rsolve : lu0;
-  const size_t gemm = (size_t)elem_size * 2 * kStage;
-  const size_t m = trunc > lu ? trunc : lu;
+  const size_t gemm = (size_t)elem_size * (2 * kStage + 64 * 64);
+  const size_t m = trunc > lu0 ? trunc : lu0;
   return m > gemm ? m : gemm;
 }
 // the tensor-core staging buffer follows the task bodies' region, 1024-aligned
@@ -1988,7 +1885,6 @@ __device__ void run_task(Ctx<T>& c, const Task& t, char* smem) {
     case TK_ROWMV: task_rowmv(c, t, smem); break;
     case TK_TRUNC: task_trunc(c, t, smem); break;
     case TK_DADD: task_dadd(c, t, smem); break;
-    case TK_RSOLVE: task_rsolve(c, t, smem); break;
     default: break;
   }
 }
@@ -2105,7 +2001,6 @@ __global__ void __launch_bounds__(NT, EXEC_MIN_BLOCKS) exec_kernel(const __grid_
       c.eps = P.eps;
       c.nrhs_slot = P.nrhs_slot;
       c.nrhs = P.nrhs;
-      c.term_p = P.term_p;
       c.alpha = P.alpha;
       run_task(c, t, smem);
     }
@@ -2231,6 +2126,144 @@ cudaError_t tc_tile_product(const float* A, const float* B, float* D, int K, int
   tc_tile_kernel<<<1, NT, tc::kTcStageBytes, s>>>(A, B, D, K, status, wait_ns);
   return cudaGetLastError();
 }
+#endif
+
+#if !HLU_EXEC_TC
+// ---------------------------------------------------------------- solve blocks
+// Dense copies of the solve blocks' diagonal blocks: one CTA per leaf block.
+template <class T>
+__global__ void __launch_bounds__(NT) k_inv_copy(const InvLeaf* leaves, T* arena, const int32_t* ranks) {
+  const InvLeaf f = leaves[blockIdx.x];
+  const int r = f.slot < 0 ? 0 : ranks[f.slot];
+  for (int64_t e = threadIdx.x; e < (int64_t)f.m * f.n; e += NT) {
+    const int i = (int)(e % f.m), j = (int)(e / f.m);
+    T s = 0;
+    if (f.slot < 0)
+      s = arena[f.off + e];
+    else
+      for (int l = 0; l < r; ++l) s += arena[f.off + i + (int64_t)l * f.m] * arena[f.off2 + j + (int64_t)l * f.n];
+    arena[f.dst + i + (int64_t)j * f.ld] = s;
+  }
+}
+
+// Products M_ik X_kj of the block substitution, k in [k, kend), as one pipeline.
+template <class T>
+struct InvCursor {
+  const InvUnit* u;  // the block's units
+  T* arena;
+  bool upper;
+  int i, j, k, kend, l0;
+  __device__ bool first() {
+    l0 = 0;
+    return k < kend;
+  }
+  __device__ bool next() {
+    l0 += KC;
+    if (l0 < u[k].rows) return true;
+    l0 = 0;
+    return ++k < kend;
+  }
+  __device__ Chunk<T> chunk() const {
+    const InvUnit &I = u[i], &J = u[j], &Q = u[k];
+    const T* A = arena + I.d_off + I.begin + (int64_t)(Q.begin + l0) * I.m;
+    const T* B = arena + (upper ? Q.u_off + (int64_t)(J.begin - Q.begin) * Q.ld : Q.l_off + (int64_t)J.begin * Q.ld) + l0;
+    return Chunk<T>{Mat<T>{A, 1, I.m}, Mat<T>{B, 1, Q.ld}, 0, I.rows, J.rows, min(KC, Q.rows - l0), 0, T(1)};
+  }
+};
+
+// Columns of unit j of the inverse of P^T L (blockIdx.y 0) or U (1) of one
+// solve block, by block substitution down or up the units: X_ij = L_i^-1 P_i
+// (I_ij - sum_k M_ik X_kj), or U_i^-1 (...).  The columns are independent, so
+// every unit of every block has its own CTA; the triangular part runs eight
+// columns per warp (one per right-hand side of the substitution), the pivot
+// tile and the right-hand sides in shared memory.
+template <class T>
+__global__ void __launch_bounds__(NT) k_inv_units(const InvUnit* units, T* arena, const int32_t* piv) {
+  extern __shared__ __align__(16) char smem[];
+  T* As = reinterpret_cast<T*>(smem);
+  T* Bs = As + kStage;
+  T* A = Bs + kStage;  // the diagonal tile, ld 64
+  T* X = A + 64 * 64;  // right-hand sides, ld 65
+  __shared__ int perm[64];
+  __shared__ T dinv[64];
+  const bool upper = blockIdx.y == 1;
+  const InvUnit* u = units + units[blockIdx.x].first;
+  const int j = (int)blockIdx.x - units[blockIdx.x].first, nu = u[0].count;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nj = u[j].rows;
+  for (int step = 0; step < (upper ? j + 1 : nu - j); ++step) {
+    const int i = upper ? j - step : j + step;
+    const InvUnit I = u[i];
+    const int n = I.rows;
+    T acc[4][4];
+    acc_zero(acc);
+    InvCursor<T> cur{u, arena, upper, i, j, upper ? i + 1 : j, upper ? j + 1 : i, 0};
+    tile_mma_seq(acc, cur, As, Bs);
+    const T* D = arena + I.d_off + I.begin + (int64_t)I.begin * I.m;
+    for (int e = threadIdx.x; e < n * n; e += NT) A[e % n + 64 * (e / n)] = __ldcg(D + e % n + (int64_t)(e / n) * I.m);
+    if (threadIdx.x < n) perm[threadIdx.x] = __ldcg(piv + I.piv_off + threadIdx.x);
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const int r = tx * 4 + p, c = ty * 4 + q;
+        X[r + 65 * c] = (i == j && r == c ? T(1) : T(0)) - acc[p][q];
+      }
+    __syncthreads();
+    if (threadIdx.x < n) dinv[threadIdx.x] = T(1) / A[threadIdx.x + 64 * threadIdx.x];
+    __syncthreads();
+    constexpr int Q = 64 / (NT / 32);
+    const int r0 = lane, r1 = lane + 32, c0 = warp * Q;
+    T v0[Q], v1[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const T* x = X + 65 * (c0 + q);
+      v0[q] = r0 < n ? x[upper ? r0 : perm[r0]] : T(0);
+      v1[q] = r1 < n ? x[upper ? r1 : perm[r1]] : T(0);
+    }
+    for (int st = 0; st < n; ++st) {
+      const int l = upper ? n - 1 - st : st;
+      // rows still to be updated; row l itself is scaled in U
+      const T a0 = (upper ? r0 < l : (r0 > l && r0 < n)) ? A[r0 + 64 * l] : T(0);
+      const T a1 = (upper ? r1 < l : (r1 > l && r1 < n)) ? A[r1 + 64 * l] : T(0);
+      const T d = upper ? dinv[l] : T(1);
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const T x = __shfl_sync(0xffffffffu, l < 32 ? v0[q] : v1[q], l & 31) * d;
+        if (upper && r0 == l) v0[q] = x;
+        if (upper && r1 == l) v1[q] = x;
+        v0[q] -= a0 * x;
+        v1[q] -= a1 * x;
+      }
+    }
+    T* out = arena + (upper ? I.u_off + (int64_t)(u[j].begin - I.begin) * I.ld : I.l_off + (int64_t)u[j].begin * I.ld);
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (c0 + q < nj) {
+        if (r0 < n) __stcg(out + r0 + (int64_t)(c0 + q) * I.ld, v0[q]);
+        if (r1 < n) __stcg(out + r1 + (int64_t)(c0 + q) * I.ld, v1[q]);
+      }
+    __syncthreads();
+  }
+}
+
+template <class T>
+cudaError_t invert_blocks(const InvUnit* units, int32_t n_units, const InvLeaf* leaves, int32_t n_leaves, T* arena,
+                          const int32_t* ranks, const int32_t* piv, cudaStream_t s) {
+  const size_t sm = sizeof(T) * (2 * kStage + 64 * 64 + 65 * 64);
+  cudaError_t e = cudaFuncSetAttribute(k_inv_units<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess || n_units == 0) return e;
+  note_launch();
+  k_inv_copy<T><<<n_leaves, NT, 0, s>>>(leaves, arena, ranks);
+  note_launch();
+  k_inv_units<T><<<dim3(n_units, 2), NT, sm, s>>>(units, arena, piv);
+  return cudaGetLastError();
+}
+template cudaError_t invert_blocks<float>(const InvUnit*, int32_t, const InvLeaf*, int32_t, float*, const int32_t*,
+                                          const int32_t*, cudaStream_t);
+template cudaError_t invert_blocks<double>(const InvUnit*, int32_t, const InvLeaf*, int32_t, double*, const int32_t*,
+                                           const int32_t*, cudaStream_t);
 #endif
 
 size_t exec_smem_bytes(int elem_size) {

@@ -26,8 +26,6 @@ struct ProbSched {
   int64_t limit;            // tasks with index >= limit are not run
   int32_t nrhs_slot;        // rank slot of the right-hand-side count, and its
   int32_t nrhs;             // value for this launch (read without a load)
-  const int32_t* term_p;    // solve launches: each term's column count, resolved
-                            // after the factorisation (-1: read it live); else null
   double alpha;             // scalar of TF_ALPHA tasks and PF_ALPHA pieces (Schulz start)
 };
 constexpr int kMaxBatch = 64;  // problems in one launch
@@ -79,6 +77,39 @@ cudaError_t exec_launch(const ExecArgs& a, int grid, cudaStream_t s);
 cudaError_t tc_tile_product(const float* A, const float* B, float* D, int K, int32_t* status,
                             unsigned long long wait_ns, cudaStream_t s);
 }  // namespace tcx
+
+// One problem of a triangular-solve launch (solve.cu).
+struct SolveProb {
+  const Task* tasks;        // in ticket order
+  const Term* terms;
+  const int32_t* term_p;    // columns of each term's A (its rank after the factorisation)
+  const int64_t* succ_ptr;
+  const int32_t* succ_idx;
+  const int32_t* indeg0;    // predecessor counts
+  int32_t* indeg;           // unfinished predecessors of the running launch
+  unsigned long long* ticket;  // next task to hand out
+  void* arena;
+  const int32_t* ranks;
+  int64_t ntasks;
+  int32_t nrhs;
+  int32_t cta0;             // first CTA that starts on this problem (set by solve_launch)
+};
+struct SolveArgs {
+  SolveProb probs[kMaxBatch];
+  int32_t nprobs;
+  int32_t* status;          // as ExecArgs::status
+  unsigned long long wait_limit_ns;
+  unsigned long long* trace;  // as ExecArgs::trace (one problem)
+};
+template <class T>
+cudaError_t solve_launch(SolveArgs& a, cudaStream_t s);
+
+// Inverts the triangular factors of every solve block of a factored arena
+// (exec.cu): dense copies of the diagonal blocks, then one CTA per unit and
+// triangle.
+template <class T>
+cudaError_t invert_blocks(const InvUnit* units, int32_t n_units, const InvLeaf* leaves, int32_t n_leaves, T* arena,
+                          const int32_t* ranks, const int32_t* piv, cudaStream_t s);
 
 constexpr int kExecThreads = 256;
 constexpr int kTruncStack = 96;  // columns of a truncation stack; wider pieces are stacked in parts

@@ -3,7 +3,7 @@
 // The scheduler derives its edges from an abstract model of the data: accesses
 // to (buffer, leaf-cluster segment) pairs, plus fences where temporary memory
 // is re-used.  This check does not use that model.  It reads only the emitted
-// tasks (operand views, ROWMV / RSOLVE terms, TRUNC pieces, pivot offsets,
+// tasks (operand views, ROWMV terms, TRUNC pieces, pivot offsets,
 // rank slots) and expands every operand to the elements it may touch: a view
 // at its full capacity, whatever rank a run produces.  It then replays the DAG
 // in program order.  An access that conflicts with an earlier one (write after
@@ -14,7 +14,7 @@
 // address spaces, and every access must stay inside its space.
 //
 // Rank slots are read where the device kernels take a live column count
-// (TRSM, PROJ, ROWMV, DADD, RSOLVE operands and the terms' and pieces' left
+// (TRSM, PROJ, ROWMV, DADD operands and the terms' and pieces' left
 // factors; the solve's right-hand-side count is a launch parameter, not a
 // slot read).  ROWMV writes its output's slot with a copy of its input's
 // count and TRUNC with the rank it computes.  Two writes of the same copied
@@ -260,18 +260,10 @@ class HazardCheck {
       case TK_TRSM_L: count(t.b); view(t.a); range(SP_PIV, t.piv_off, t.a.rows); view(t.b); break;
       case TK_TRSM_UT:
       case TK_TRSM_U: count(t.b); view(t.a); view(t.b); break;
-      case TK_PROJ: count(t.a); count(t.b); view(t.a); view(t.b); break;
+      case TK_PROJ: count(t.a); count(t.b); view(t.a); view(t.b); if (t.flags & TF_ADD) view(t.c); break;
       case TK_ROWMV: count(t.b); terms(t); if (!(t.flags & TF_OVERWRITE)) view(t.c); break;
       case TK_TRUNC: pieces(t); break;
       case TK_DADD: count(t.c); count(t.a); view(t.a); view(t.b); if (!(t.flags & TF_OVERWRITE)) view(t.c); break;
-      case TK_RSOLVE:
-        count(t.b);
-        count(t.c);
-        terms(t);
-        view(t.a);
-        if (!(t.flags & TF_UPPER)) range(SP_PIV, t.piv_off, t.a.rows);
-        view(t.c);
-        break;
       case TK_FENCE: break;
       default: throw std::logic_error("task type");
     }
@@ -285,7 +277,6 @@ class HazardCheck {
       case TK_ROWMV: view(t.c); break;
       case TK_TRUNC: view(t.a); view(t.b); break;
       case TK_DADD: view(t.c); break;
-      case TK_RSOLVE: view(t.c); break;
       default: break;
     }
     writing_ = false;

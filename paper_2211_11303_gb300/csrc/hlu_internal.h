@@ -18,6 +18,9 @@ struct Block {
 };
 enum { KIND_ADM = 0, KIND_DENSE = 1, KIND_SUB = 2 };
 
+// Largest diagonal block whose triangular factors are inverted for the solve.
+constexpr int32_t kSolveBlock = 512;
+
 // Largest (and default) rank capacity of an admissible block.
 constexpr int32_t kRankMax = 64;
 
@@ -43,20 +46,20 @@ enum TaskType : int32_t {
   TK_ROWMV = 5,   // c (n x k) <- [c] + sign * sum_terms A_t B_t
   TK_TRUNC = 6,   // (a, b) <- truncate(sum_pieces sign X Y^T) to eps, rank -> out_slot
   TK_DADD = 7,    // c (m x n) <- [c] + sign * a b^T  (a: m x k, b: n x k)
-  TK_RSOLVE = 8,  // c <- tri(a)^-1 (c - sum_terms A_t B_t): one tile of a triangular solve;
-                  // flags & TF_UPPER: U^-1, else L^-1 P (pivots at piv_off)
+  // 8: no longer used (its row of the executor's profile stays, empty)
   TK_NUM = 9,
   TK_FENCE = 9    // no work: orders re-use of temporary memory after its readers
 };
 // TF_ALPHA (DADD) and PF_ALPHA (a TRUNC piece): the sign is multiplied by the
-// launch's scalar alpha (the Schulz start X_0 = alpha A)
-enum : int32_t { TF_OVERWRITE = 1, TF_UPPER = 2, TF_ALPHA = 4 };
+// launch's scalar alpha (the Schulz start X_0 = alpha A).  TF_ADD (PROJ of the
+// triangular solve): c += a^T b instead of c = a^T b.
+enum : int32_t { TF_OVERWRITE = 1, TF_ALPHA = 4, TF_ADD = 8 };
 enum : int32_t { PF_ALPHA = 1 };
 
 struct Task {
   int32_t type;
   int32_t flags;
-  int32_t list_begin, list_count;  // ROWMV / RSOLVE terms or TRUNC pieces
+  int32_t list_begin, list_count;  // ROWMV terms or TRUNC pieces
   View a, b, c;
   int64_t piv_off;   // pivot vector offset (int32 elements) for leaf tasks
   int32_t out_slot;  // rank slot written by the task (-1: none)
@@ -91,6 +94,26 @@ struct Schedule {
   int64_t n_edges = 0;
 };
 
+// One unit (tile-level cluster) of a solve block: the triangular solve works
+// with the explicit inverses of the diagonal blocks of clusters of up to
+// kSolveBlock DOFs, kept as one row panel per unit.  With m the block's size,
+// the unit's rows [begin, begin + rows) of (P^T L)^-1 have begin + rows columns,
+// those of U^-1 the columns from begin on (m - begin); both column-major with
+// leading dimension ld.
+struct InvUnit {
+  int64_t l_off, u_off;  // the two row panels
+  int64_t d_off;         // the block's dense copy (m x m, ld m; scratch in the ring)
+  int64_t piv_off;       // pivots of the unit's diagonal tile
+  int32_t ld, begin, rows, m;
+  int32_t first, count;  // the block's units
+};
+// A leaf block of a solve block's diagonal block, copied into its dense copy.
+struct InvLeaf {
+  int64_t off, off2;     // dense tile, or X and Y of a low-rank block
+  int64_t dst;           // element (0, 0) in the dense copy
+  int32_t m, n, ld, slot;  // slot < 0: dense
+};
+
 // Layout of one problem's factor arena (element offsets).
 struct ArenaLayout {
   int64_t total = 0;       // elements
@@ -111,6 +134,9 @@ struct ArenaLayout {
   int32_t wmax = 0;                // largest stacked width of a TRUNC
   int64_t ring_off = 0, ring_size = 0;  // region for temporaries
   int64_t out_off = -1;            // H-matrix apply: output vector (N x nrhs_max), -1 if none
+  int64_t z_off = -1;              // triangular solve: forward result (N x nrhs_max)
+  std::vector<InvUnit> inv_units;  // inverted diagonal blocks of the triangular solve
+  std::vector<InvLeaf> inv_leaves;
 };
 
 struct SchedStats {

@@ -109,7 +109,7 @@ void h_proj(HostCtx<T>& c, const Task& t) {
     for (int j = 0; j < k; ++j) {
       T s = 0;
       for (int l = 0; l < m; ++l) s += at(c, t.a, l, i) * at(c, t.b, l, j);
-      at(c, t.c, i, j) = s;
+      at(c, t.c, i, j) = (t.flags & TF_ADD) ? at(c, t.c, i, j) + s : s;
     }
 }
 
@@ -354,19 +354,6 @@ void h_trunc(HostCtx<T>& c, const Task& t) {
 }
 
 template <class T>
-void h_rsolve(HostCtx<T>& c, const Task& t) {
-  Task r = t;
-  r.type = TK_ROWMV;
-  r.flags = 0;
-  r.out_slot = -1;
-  h_rowmv(c, r);
-  Task s = t;
-  s.type = (t.flags & TF_UPPER) ? TK_TRSM_U : TK_TRSM_L;
-  s.b = t.c;
-  h_trsm(c, s);
-}
-
-template <class T>
 void run_task(HostCtx<T>& c, const Task& t) {
   switch (t.type) {
     case TK_GETRF: h_getrf(c, t); break;
@@ -377,7 +364,6 @@ void run_task(HostCtx<T>& c, const Task& t) {
     case TK_ROWMV: h_rowmv(c, t); break;
     case TK_TRUNC: h_trunc(c, t); break;
     case TK_DADD: h_dadd(c, t); break;
-    case TK_RSOLVE: h_rsolve(c, t); break;
     case TK_FENCE: break;
     default: throw std::logic_error("task type");
   }
@@ -437,6 +423,58 @@ int host_execute(const Schedule& S, T* arena, int32_t* ranks, int32_t* piv, doub
   if (cap_hits) *cap_hits += c.cap_hits;
   return c.status;
 }
+
+// The row panels of (P^T L)^-1 and U^-1 of every solve block, column by column
+// by block substitution over the block's dense copy.
+template <class T>
+void host_invert(const ArenaLayout& L, T* arena, const int32_t* ranks, const int32_t* piv) {
+  for (const InvLeaf& f : L.inv_leaves)
+    for (int32_t j = 0; j < f.n; ++j)
+      for (int32_t i = 0; i < f.m; ++i) {
+        T s = 0;
+        if (f.slot < 0)
+          s = arena[f.off + i + (int64_t)j * f.m];
+        else
+          for (int32_t l = 0; l < ranks[f.slot]; ++l)
+            s += arena[f.off + i + (int64_t)l * f.m] * arena[f.off2 + j + (int64_t)l * f.n];
+        arena[f.dst + i + (int64_t)j * f.ld] = s;
+      }
+  for (size_t b = 0; b < L.inv_units.size(); b += L.inv_units[b].count) {
+    const InvUnit* u = &L.inv_units[b];
+    const int32_t nu = u[0].count, m = u[0].m;
+    const T* D = arena + u[0].d_off;
+    std::vector<T> x(m), y(64);
+    for (int32_t c = 0; c < m; ++c) {
+      std::fill(x.begin(), x.end(), T(0));
+      for (int32_t q = 0; q < nu; ++q) {  // P^T L, first unit down
+        if (u[q].begin + u[q].rows <= c) continue;
+        const int32_t n = u[q].rows, r0 = u[q].begin;
+        const int32_t* p = piv + u[q].piv_off;
+        y.assign(n, T(0));
+        for (int32_t i = 0; i < n; ++i) {
+          T s = r0 + p[i] == c ? T(1) : T(0);
+          for (int32_t k = 0; k < r0; ++k) s -= D[r0 + p[i] + (int64_t)k * m] * x[k];
+          for (int32_t k = 0; k < i; ++k) s -= D[r0 + i + (int64_t)(r0 + k) * m] * y[k];
+          y[i] = s;
+        }
+        for (int32_t i = 0; i < n; ++i) arena[u[q].l_off + i + (int64_t)c * u[q].ld] = x[r0 + i] = y[i];
+      }
+      std::fill(x.begin(), x.end(), T(0));
+      for (int32_t q = nu - 1; q >= 0; --q) {  // U, last unit up
+        if (u[q].begin > c) continue;
+        const int32_t n = u[q].rows, r0 = u[q].begin;
+        for (int32_t i = r0 + n - 1; i >= r0; --i) {
+          T s = i == c ? T(1) : T(0);
+          for (int32_t k = i + 1; k < m; ++k) s -= D[i + (int64_t)k * m] * x[k];
+          x[i] = s / D[i + (int64_t)i * m];
+          arena[u[q].u_off + (i - r0) + (int64_t)(c - r0) * u[q].ld] = x[i];
+        }
+      }
+    }
+  }
+}
+template void host_invert<double>(const ArenaLayout&, double*, const int32_t*, const int32_t*);
+template void host_invert<float>(const ArenaLayout&, float*, const int32_t*, const int32_t*);
 
 template int host_execute<double>(const Schedule&, double*, int32_t*, int32_t*, double, uint64_t,
                                   int32_t*, int64_t, double);

@@ -14,8 +14,12 @@
 // capacities; kernels read the live rank from a rank slot when they run.
 #include <algorithm>
 #include <chrono>
+#include <cstdlib>
 #include <cstring>
+#include <functional>
+#include <queue>
 #include <stdexcept>
+#include <utility>
 
 #include "hlu_internal.h"
 
@@ -373,29 +377,6 @@ class Sched {
     end();
   }
   void trsm_leaf(int32_t type, int32_t d, const MV& V) {
-    const int32_t sg = seg_begin_[rowc(d)];
-    if ((type == TK_TRSM_L || type == TK_TRSM_U) && seg_end_[rowc(d)] - sg == 1 && sg < (int32_t)pending_.size() &&
-        pending_[sg].active && seg_cluster_[sg] == rowc(d)) {
-      // the late update of this segment and its triangular solve in one task
-      Pending& pd = pending_[sg];
-      Task k = make(TK_RSOLVE);
-      k.flags = type == TK_TRSM_U ? TF_UPPER : 0;
-      k.a = mvD(d).v;
-      k.b = pd.Vin.v;  // column count source
-      k.c = V.v;
-      k.piv_off = L_.piv_off[d];
-      k.sign = pd.sign;
-      k.list_begin = (int32_t)S_->terms.size();
-      k.list_count = (int32_t)pd.list.size();
-      begin(k);
-      push_terms(pd.lv, pd.T, pd.list, pd.Vin, rowc(d), pd.trans);
-      acc_rank(pd.Vin);
-      acc(mvD(d), false);
-      acc(V, true);
-      end();
-      pd = Pending();
-      return;
-    }
     Task t = make(type);
     t.a = mvD(d).v;
     t.b = V.v;
@@ -418,15 +399,13 @@ class Sched {
   // Vout (+)= sign * op(b) Vin, op = transpose when trans.  Vin covers the
   // in-cluster of b, Vout its out-cluster.  overwrite: Vout starts from zero
   // and out_slot receives Vin's column count.
-  // late_seg >= 0 (solves, accumulating): the terms of every output unit are
-  // split into two ROWMV tasks, those whose input does not cover segment
-  // late_seg (the input's last segment to be solved) first, so that only the
-  // few terms reading it wait for the end of the preceding solve.
-  // fuse_seg >= 0 (solve schedule): the late task of the unit that is
-  // segment fuse_seg is not emitted here but merged into that segment's next
-  // triangular leaf solve (one RSOLVE task instead of a ROWMV and a TRSM).
-  void hmul(int32_t b, const MV& Vin, const MV& Vout, float sign, bool trans, bool overwrite,
-            int32_t out_slot, int32_t late_seg = -1, int32_t fuse_seg = -1) {
+  // late_seg >= 0 (accumulating): the terms of every output unit are split
+  // into ROWMV tasks by how long before late_seg, the input's last segment
+  // to be solved, their input is final: group 0 reads late_seg itself, group
+  // g >= 1 segments 2^(g-1) to 2^g - 1 before it.  Far groups run first, so
+  // only the few terms reading late_seg wait for the end of the preceding solve.
+  void hmul(int32_t b, const MV& Vin, const MV& Vout, float sign, bool trans, bool overwrite, int32_t out_slot,
+            int32_t late_seg = -1) {
     std::vector<int32_t> lv;
     leaves_of(b, lv);
     int32_t oc = trans ? colc(b) : rowc(b);
@@ -482,50 +461,20 @@ class Sched {
     MV kview = Vin;
     for (int32_t l = 0; l < nu; ++l) {
       if (cnt[l] == cnt[l + 1] && !overwrite) continue;
-      const int32_t lc = units[l];
-      // terms grouped by how long before late_seg their input is final: group
-      // g >= 1 holds the terms whose last-solved input segment lies between
-      // 2^(g-1) and 2^g - 1 segments before late_seg, group 0 those reading
-      // late_seg itself; the groups run in that order, so each one waits only
-      // for inputs solved well before it and the last ones are small
       constexpr int kGroups = 33;
       std::vector<int32_t> parts[kGroups];
       for (int32_t q = cnt[l]; q < cnt[l + 1]; ++q) {
-        const int32_t i = items[q];
         int g = 0;
-        if (late_seg >= 0 && !overwrite) {
-          const int32_t ic = trans ? rowc(lv[i]) : colc(lv[i]);
-          int32_t dist = 0;
-          if (late_seg >= seg_end_[ic])
-            dist = late_seg - (seg_end_[ic] - 1);
-          else if (late_seg < seg_begin_[ic])
-            dist = seg_begin_[ic] - late_seg;
-          while (dist > 0) {
-            ++g;
-            dist >>= 1;
-          }
-        }
-        parts[g].push_back(i);
+        if (late_seg >= 0 && !overwrite)
+          for (int32_t dist = late_seg - (seg_end_[colc(lv[items[q]])] - 1); dist > 0; dist >>= 1) ++g;
+        parts[g].push_back(items[q]);
       }
-      for (int part = kGroups - 1; part >= 0; --part) {
-        if (parts[part].empty() && (part != 0 || !overwrite)) continue;
-        if (part == 0 && late_seg >= 0 && fuse_seg >= 0 && fuse_seg < (int32_t)pending_.size() &&
-            lc == seg_cluster_[fuse_seg] && !pending_[fuse_seg].active) {
-          Pending& pd = pending_[fuse_seg];
-          pd.active = true;
-          pd.lv = lv;
-          pd.T = T;
-          pd.list = parts[part];
-          pd.Vin = Vin;
-          pd.sign = sign;
-          pd.trans = trans;
-          continue;
-        }
-        emit_rowmv(lv, T, parts[part], Vin, Vout, lc, sign, trans, overwrite, out_slot, kview);
-      }
+      for (int part = kGroups - 1; part >= 0; --part)
+        if (!parts[part].empty() || (part == 0 && overwrite))
+          emit_rowmv(lv, T, parts[part], Vin, Vout, units[l], sign, trans, overwrite, out_slot, kview);
     }
   }
-  // the terms of a ROWMV (or RSOLVE) task for unit lc, with their reads
+  // the terms of a ROWMV task for unit lc, with their reads
   void push_terms(const std::vector<int32_t>& lv, const std::vector<MV>& T, const std::vector<int32_t>& list,
                   const MV& Vin, int32_t lc, bool trans) {
     for (int32_t i : list) {
@@ -590,7 +539,7 @@ class Sched {
     const Cluster& c = C_[rowc(d)];
     MV V0 = sub(V, c.son[0]), V1 = sub(V, c.son[1]);
     solve_lower(son(d, 0, 0), V0);
-    hmul(son(d, 1, 0), V0, V1, -1.0f, false, false, -1, seg_end_[c.son[0]] - 1, seg_begin_[c.son[1]]);
+    hmul(son(d, 1, 0), V0, V1, -1.0f, false, false, -1, seg_end_[c.son[0]] - 1);
     solve_lower(son(d, 1, 1), V1);
   }
   void solve_upperT(int32_t d, const MV& W) {
@@ -604,18 +553,6 @@ class Sched {
     hmul(son(d, 0, 1), W0, W1, -1.0f, true, false, -1);
     solve_upperT(son(d, 1, 1), W1);
   }
-  void solve_upper(int32_t d, const MV& V) {
-    if (kind(d) == KIND_DENSE) {
-      trsm_leaf(TK_TRSM_U, d, V);
-      return;
-    }
-    const Cluster& c = C_[rowc(d)];
-    MV V0 = sub(V, c.son[0]), V1 = sub(V, c.son[1]);
-    solve_upper(son(d, 1, 1), V1);
-    hmul(son(d, 0, 1), V1, V0, -1.0f, false, false, -1, seg_begin_[c.son[1]], seg_end_[c.son[0]] - 1);
-    solve_upper(son(d, 0, 0), V0);
-  }
-
   // ---------------------------------------------------------------- truncation
   void emit_trunc(const MV& X, const MV& Y, int32_t slot, int32_t cap,
                   const std::vector<PieceMV>& ps, bool alpha = false) {
@@ -887,15 +824,144 @@ class Sched {
     lu(d11);
   }
 
+  // ---------------------------------------------------------------- the solve of step III
+  // x = U^-1 (L^-1 P w).  The chain through the diagonal runs over solve
+  // blocks (clusters of up to kSolveBlock DOFs) instead of tiles: a block is
+  // one parallel step, its units multiplied by their row panels of the
+  // inverted triangular factor (overwriting ROWMV tasks).  w and x share the
+  // work vector, the forward result has its own (z).
   void solve_all(int32_t nrhs_max) {
-    pending_.assign(seg_cluster_.size(), Pending());
-    MV W;
-    W.buf = new_buf_leaves(0);  // per-segment tracking over the whole vector
-    W.clus = 0;
-    int32_t N = sz(0);
-    W.v = View{L_.work_off, 1, N, N, nrhs_max, L_.nrhs_slot, 0};
-    solve_lower(0, W);
-    solve_upper(0, W);
+    const int32_t N = sz(0);
+    W_.buf = new_buf_leaves(0);  // per-segment tracking over the whole vector
+    Z_.buf = new_buf_leaves(0);
+    W_.clus = Z_.clus = 0;
+    W_.v = View{L_.work_off, 1, N, N, nrhs_max, L_.nrhs_slot, 0};
+    Z_.v = View{L_.z_off, 1, N, N, nrhs_max, L_.nrhs_slot, 0};
+    if (L_.inv_units.size() != seg_cluster_.size()) throw std::logic_error("solve units are not the segments");
+    blk_of_seg_.clear();
+    for (const InvUnit& u : L_.inv_units) blk_of_seg_.push_back(u.first);
+    for (int32_t k = 0, last = -1, id = -1; k < (int32_t)blk_of_seg_.size(); ++k) {
+      if (blk_of_seg_[k] != last) ++id;
+      last = blk_of_seg_[k];
+      blk_of_seg_[k] = id;
+    }
+    solve_diag(0, true);
+    solve_diag(0, false);
+  }
+  void solve_diag(int32_t d, bool fwd) {
+    const Cluster& c = C_[rowc(d)];
+    if (kind(d) == KIND_DENSE || c.size <= kSolveBlock) {
+      for (int32_t q = seg_begin_[rowc(d)]; q < seg_end_[rowc(d)]; ++q) inv_unit(q, fwd);
+      return;
+    }
+    solve_diag(son(d, fwd ? 0 : 1, fwd ? 0 : 1), fwd);
+    solve_update(fwd ? son(d, 1, 0) : son(d, 0, 1), fwd);
+    solve_diag(son(d, fwd ? 1 : 0, fwd ? 1 : 0), fwd);
+  }
+  // rows of one unit of its block's inverse times the block's right-hand side
+  void inv_unit(int32_t q, bool fwd) {
+    const InvUnit& u = L_.inv_units[q];
+    const MV& in = fwd ? W_ : Z_;
+    const MV out = sub(fwd ? Z_ : W_, seg_cluster_[q]);
+    const int32_t s0 = fwd ? u.first : q, s1 = fwd ? q + 1 : u.first + u.count;
+    const int32_t cols = fwd ? u.begin + u.rows : u.m - u.begin;
+    Term tm;
+    std::memset(&tm, 0, sizeof(tm));
+    tm.A = View{fwd ? u.l_off : u.u_off, 1, u.ld, u.rows, cols, -1, 0};
+    tm.B = in.v;
+    tm.B.off += C_[seg_cluster_[s0]].off;
+    tm.B.rows = cols;
+    Task k = make(TK_ROWMV);
+    k.flags = TF_OVERWRITE;
+    k.c = out.v;
+    k.b = in.v;  // column count source
+    k.list_begin = (int32_t)S_->terms.size();
+    k.list_count = 1;
+    grow4(S_->terms);
+    S_->terms.push_back(tm);
+    begin(k);
+    for (int32_t s = s0; s < s1; ++s) acc(sub(in, seg_cluster_[s]), false);
+    acc(out, true);
+    end();
+  }
+  // out -= H(b) in for an off-diagonal block, in solved before out.  Terms and
+  // projections are grouped by how many solve blocks before the last one of
+  // the input they are final (group 0 the last block, group g blocks 2^(g-1)
+  // to 2^g - 1 before it) and run far groups first, so that little work
+  // waits for the last block.  Output units solved kMergeBlocks or more blocks
+  // later have time: all their terms go into one task.
+  void solve_update(int32_t b, bool fwd) {
+    constexpr int32_t kMergeBlocks = 2;
+    const MV in = sub(fwd ? Z_ : W_, colc(b)), out = sub(fwd ? W_ : Z_, rowc(b));
+    std::vector<int32_t> lv;
+    leaves_of(b, lv);
+    const int32_t last = fwd ? blk_of_seg_[seg_end_[colc(b)] - 1] : blk_of_seg_[seg_begin_[colc(b)]];
+    auto group = [&](int32_t seg) {
+      int g = 0;
+      for (int32_t dist = std::abs(blk_of_seg_[seg] - last); dist > 0; dist >>= 1) ++g;
+      return g;
+    };
+    std::vector<MV> T(lv.size());
+    for (size_t i = 0; i < lv.size(); ++i) {
+      const int32_t be = lv[i];
+      if (kind(be) != KIND_ADM) continue;
+      const MV A = mvY(be), vin = sub(in, colc(be));
+      const int32_t cap = L_.cap[be];
+      MV t;
+      t.clus = -1;
+      const int64_t toff = alloc((int64_t)cap * std::max(vin.v.cols, 1));
+      t.buf = new_buf_single();
+      bind_alloc(t.buf);
+      t.v = View{toff, 1, cap, cap, vin.v.cols, vin.v.slot, 0};
+      // one task per run of segments of the same group, the farthest first
+      const int32_t s0 = seg_begin_[colc(be)], s1 = seg_end_[colc(be)];
+      bool add = false;
+      for (int32_t done = 0; done < s1 - s0;) {
+        int32_t n = 1;
+        auto at = [&](int32_t k) { return fwd ? s0 + k : s1 - 1 - k; };
+        while (done + n < s1 - s0 && group(at(done + n)) == group(at(done))) ++n;
+        const int32_t lo = std::min(at(done), at(done + n - 1)), hi = lo + n;
+        const bool whole = n == s1 - s0;  // (a column cluster inside one segment has no segment of its own)
+        const int32_t r0 = whole ? 0 : C_[seg_cluster_[lo]].off - C_[colc(be)].off;
+        const int32_t r1 = whole ? sz(colc(be))
+                                 : C_[seg_cluster_[hi - 1]].off + sz(seg_cluster_[hi - 1]) - C_[colc(be)].off;
+        Task k = make(TK_PROJ);
+        k.flags = add ? TF_ADD : 0;
+        k.a = A.v;
+        k.b = vin.v;
+        k.c = t.v;
+        k.a.off += r0;
+        k.b.off += r0;
+        k.a.rows = k.b.rows = r1 - r0;
+        begin(k);
+        if (whole)
+          acc(vin, false);
+        else
+          for (int32_t s = lo; s < hi; ++s) acc(sub(in, seg_cluster_[s]), false);
+        touch(bufs_[t.buf].seg0, true);
+        end();
+        add = true;
+        done += n;
+      }
+      T[i] = t;
+    }
+    const int32_t u0 = seg_begin_[rowc(b)], nu = seg_end_[rowc(b)] - u0;
+    std::vector<std::vector<int32_t>> items(nu);
+    for (size_t i = 0; i < lv.size(); ++i)
+      for (int32_t q = seg_begin_[rowc(lv[i])]; q < seg_end_[rowc(lv[i])]; ++q) items[q - u0].push_back((int32_t)i);
+    const int32_t first = fwd ? blk_of_seg_[u0] : blk_of_seg_[u0 + nu - 1];
+    constexpr int kGroups = 33;
+    for (int32_t l = 0; l < nu; ++l) {
+      const int32_t unit = nu == 1 ? rowc(b) : seg_cluster_[u0 + l];
+      const bool merge = std::abs(blk_of_seg_[u0 + l] - first) >= kMergeBlocks;
+      std::vector<int32_t> parts[kGroups];
+      for (int32_t i : items[l]) {
+        const int32_t ic = colc(lv[i]);
+        parts[merge ? 0 : group(fwd ? seg_end_[ic] - 1 : seg_begin_[ic])].push_back(i);
+      }
+      for (int g = kGroups - 1; g >= 0; --g)
+        if (!parts[g].empty()) emit_rowmv(lv, T, parts[g], in, out, unit, -1.0f, false, false, -1, in);
+    }
   }
 
  private:
@@ -937,16 +1003,8 @@ class Sched {
   std::vector<int32_t> stamp_;
   std::vector<int32_t> deps_;
   int32_t cur_ = -1;
-  // late updates waiting to be merged into a segment's leaf solve
-  struct Pending {
-    bool active = false;
-    std::vector<int32_t> lv, list;
-    std::vector<MV> T;
-    MV Vin;
-    float sign = 0;
-    bool trans = false;
-  };
-  std::vector<Pending> pending_;
+  MV W_, Z_;                        // the solve's work vector and forward result
+  std::vector<int32_t> blk_of_seg_;  // solve block of each segment, in order
 };
 
 }  // namespace
@@ -985,6 +1043,157 @@ std::vector<Block> factor_tree(const std::vector<Cluster>& C, const std::vector<
   Rec::go(C, B, tile, 0, -1, out);
   return out;
 }
+
+namespace {
+
+// The solve blocks (diagonal blocks of up to kSolveBlock DOFs, or single
+// tiles) with the storage of their inverses; d_off and dst are relative to the
+// scratch.  Returns the scratch's size.
+template <class Alloc>
+int64_t plan_inverses(const std::vector<Cluster>& C, const std::vector<Block>& B, ArenaLayout& L, Alloc& alloc) {
+  int64_t scratch = 0;
+  struct Rec {
+    const std::vector<Cluster>& C;
+    const std::vector<Block>& B;
+    ArenaLayout& L;
+    Alloc& alloc;
+    int64_t& scratch;
+    void leaves(int32_t b, int32_t off, int32_t ld, int64_t d0) {
+      const Block& k = B[b];
+      if (k.kind == KIND_SUB) {
+        for (int32_t s : k.son) leaves(s, off, ld, d0);
+        return;
+      }
+      InvLeaf f;
+      f.dst = d0 + (C[k.row].off - off) + (int64_t)(C[k.col].off - off) * ld;
+      f.m = C[k.row].size;
+      f.n = C[k.col].size;
+      f.ld = ld;
+      f.slot = k.kind == KIND_ADM ? L.slot[b] : -1;
+      f.off = k.kind == KIND_ADM ? L.x_off[b] : L.dense_off[b];
+      f.off2 = k.kind == KIND_ADM ? L.y_off[b] : -1;
+      L.inv_leaves.push_back(f);
+    }
+    void units(int32_t b, int32_t off, int32_t m, int64_t d0) {
+      const Block& k = B[b];
+      if (k.kind == KIND_SUB) {
+        units(k.son[0], off, m, d0);
+        units(k.son[3], off, m, d0);
+        return;
+      }
+      InvUnit u;
+      u.d_off = d0;
+      u.piv_off = L.piv_off[b];
+      u.begin = C[k.row].off - off;
+      u.rows = C[k.row].size;
+      u.m = m;
+      u.ld = (u.rows + 3) & ~3;
+      u.l_off = alloc((int64_t)u.ld * (u.begin + u.rows));
+      u.u_off = alloc((int64_t)u.ld * (m - u.begin));
+      L.inv_units.push_back(u);
+    }
+    void go(int32_t b) {
+      const Block& k = B[b];
+      const int32_t m = C[k.row].size;
+      if (k.kind == KIND_SUB && m > kSolveBlock) {
+        go(k.son[0]);
+        go(k.son[3]);
+        return;
+      }
+      const int32_t first = (int32_t)L.inv_units.size();
+      const int64_t d0 = scratch;
+      scratch += ((int64_t)m * m + 31) & ~int64_t(31);
+      leaves(b, C[k.row].off, m, d0);
+      units(b, C[k.row].off, m, d0);
+      for (size_t q = first; q < L.inv_units.size(); ++q) {
+        L.inv_units[q].first = first;
+        L.inv_units[q].count = (int32_t)L.inv_units.size() - first;
+      }
+    }
+  };
+  Rec r{C, B, L, alloc, scratch};
+  r.go(0);
+  return scratch;
+}
+
+// Renumbers the solve's tasks in the order in which a list scheduling with
+// kWorkers workers starts them (priority: the longest path to the end), the
+// order in which the solve kernel hands them out.  Every task starts after its
+// predecessors ended, so the order is topological.  The durations are rough
+// (microseconds): a hop and the time to read the operands.
+void order_for_tickets(Schedule& S) {
+  constexpr int kWorkers = 512;
+  const int64_t n = (int64_t)S.tasks.size();
+  if (n < 2) return;
+  std::vector<float> dur(n), prio(n, 0.0f);
+  for (int64_t t = 0; t < n; ++t) {
+    const Task& k = S.tasks[t];
+    float elems = 0;
+    if (k.type == TK_PROJ)
+      elems = (float)k.a.rows * std::min(k.a.cols, 12);
+    else
+      for (int32_t q = 0; q < k.list_count; ++q) {
+        const View& A = S.terms[k.list_begin + q].A;
+        elems += (float)A.rows * (A.slot >= 0 ? std::min(A.cols, 12) : A.cols);
+      }
+    dur[t] = 3.0f + elems * 1e-4f;
+  }
+  std::vector<int64_t> sp(n + 1, 0);
+  std::vector<int32_t> si(S.pred_idx.size()), left(n);
+  for (int64_t t = 0; t < n; ++t) {
+    left[t] = (int32_t)(S.pred_ptr[t + 1] - S.pred_ptr[t]);
+    for (int64_t e = S.pred_ptr[t]; e < S.pred_ptr[t + 1]; ++e) ++sp[S.pred_idx[e] + 1];
+  }
+  for (int64_t t = 0; t < n; ++t) sp[t + 1] += sp[t];
+  std::vector<int64_t> fill(sp.begin(), sp.end() - 1);
+  for (int64_t t = 0; t < n; ++t)
+    for (int64_t e = S.pred_ptr[t]; e < S.pred_ptr[t + 1]; ++e) si[fill[S.pred_idx[e]]++] = (int32_t)t;
+  for (int64_t t = n - 1; t >= 0; --t) {
+    for (int64_t e = sp[t]; e < sp[t + 1]; ++e) prio[t] = std::max(prio[t], prio[si[e]]);
+    prio[t] += dur[t];
+  }
+  typedef std::pair<float, int32_t> Item;
+  std::priority_queue<Item> ready;                                              // by priority, then index
+  std::priority_queue<Item, std::vector<Item>, std::greater<Item>> running;     // by end time
+  for (int64_t t = 0; t < n; ++t)
+    if (left[t] == 0) ready.push(Item(prio[t], -(int32_t)t));
+  std::vector<int32_t> order;
+  order.reserve(n);
+  float now = 0;
+  while ((int64_t)order.size() < n) {
+    while (!ready.empty() && running.size() < kWorkers) {
+      const int32_t t = -ready.top().second;
+      ready.pop();
+      order.push_back(t);
+      running.push(Item(now + dur[t], t));
+    }
+    if (running.empty()) throw std::logic_error("the solve schedule has a cycle");
+    const int32_t t = running.top().second;
+    now = running.top().first;
+    running.pop();
+    for (int64_t e = sp[t]; e < sp[t + 1]; ++e)
+      if (--left[si[e]] == 0) ready.push(Item(prio[si[e]], -si[e]));
+  }
+  std::vector<int32_t> rank(n);
+  for (int64_t k = 0; k < n; ++k) rank[order[k]] = (int32_t)k;
+  std::vector<Task> tasks(n);
+  std::vector<int64_t> pp(1, 0);
+  std::vector<int32_t> pi;
+  pi.reserve(S.pred_idx.size());
+  for (int64_t k = 0; k < n; ++k) {
+    const int32_t t = order[k];
+    tasks[k] = S.tasks[t];
+    const size_t at = pi.size();
+    for (int64_t e = S.pred_ptr[t]; e < S.pred_ptr[t + 1]; ++e) pi.push_back(rank[S.pred_idx[e]]);
+    std::sort(pi.begin() + at, pi.end());
+    pp.push_back((int64_t)pi.size());
+  }
+  S.tasks.swap(tasks);
+  S.pred_ptr.swap(pp);
+  S.pred_idx.swap(pi);
+}
+
+}  // namespace
 
 void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bfull, int32_t rank_cap,
                      int32_t nrhs_max, int32_t tile, ArenaLayout& L,
@@ -1035,6 +1244,8 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bf
   L.nrhs_max = nrhs_max;
   L.nrhs_slot = L.n_slots++;
   L.work_off = alloc((int64_t)C[0].size * nrhs_max);
+  L.z_off = alloc((int64_t)C[0].size * nrhs_max);
+  const int64_t inv_scratch = plan_inverses(C, B, L, alloc);
   L.wmax = 0;
   // ring region for temporaries (both schedules; they never run concurrently).
   // Every wrap of the ring orders the new occupants of a chunk after all
@@ -1042,10 +1253,15 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bf
   // temporaries are twice those of capacity 32, and a 2^31-element bound
   // keeps the number of wraps (and fences) of the larger workloads at what a
   // 2^30 bound gave at capacity 32.
-  const int64_t ring = std::min<int64_t>(std::max<int64_t>(8 * fe, int64_t(1) << 22), int64_t(1) << 31);
+  const int64_t ring =
+      std::max(inv_scratch, std::min<int64_t>(std::max<int64_t>(8 * fe, int64_t(1) << 22), int64_t(1) << 31));
   const int64_t ring_off = alloc(ring);
   L.ring_off = ring_off;
   L.ring_size = ring;
+  // the dense copies are scratch between the factorisation and the solves:
+  // they use the ring's memory
+  for (InvUnit& u : L.inv_units) u.d_off += ring_off;
+  for (InvLeaf& f : L.inv_leaves) f.dst += ring_off;
   const int32_t segsz = std::max(leafmax, tile);
   factor = Schedule();
   solve = Schedule();
@@ -1061,6 +1277,7 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bf
     s.solve_all(nrhs_max);
     st.temp_elems += s.temp_elems_;
   }
+  order_for_tickets(solve);
   factor.n_edges = (int64_t)factor.pred_idx.size();
   solve.n_edges = (int64_t)solve.pred_idx.size();
   st.n_factor_tasks = (int64_t)factor.tasks.size();

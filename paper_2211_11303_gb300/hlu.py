@@ -122,6 +122,7 @@ SIGNATURES = {
     "hlu_debug_host_factor_solve": (_i32, [_i32, _vp, _i32, _vp, _vp, _vp, _vp, _vp, _f64, _i32,
                                            _i32, _i32, ctypes.c_uint64, _i32, _vp, _vp, _vp]),
     "hlu_debug_wait_timeout": (_i32, [_f64, _vp]),
+    "hlu_debug_solve_wait_timeout": (_i32, [_f64, _vp]),
     "hlu_debug_host_hinverse": (_i32, [_i32, _vp, _i32, _vp, _vp, _vp, _vp, _vp, _f64, _i32, _i32, _f64, _i32,
                                        _i32, _vp, _vp, _vp]),
     "hlu_debug_host_factor_prefix": (_i32, [_i32, _vp, _i32, _vp, _vp, _vp, _vp, _vp, _f64, _i32, _i32, _i32,
