@@ -137,7 +137,7 @@ typedef struct {
   int32_t n_clusters, n_blocks, n_adm, n_dense;
   int32_t rank_wanted_max;  /* largest rank a truncation asked for (s_i > eps s_1);
                                rank capacity + 1 when it asked for more          */
-  int32_t trunc_dense_fallbacks; /* dense-route truncations redone by the stack route */
+  int32_t trunc_dense_fallbacks; /* dense- or sampled-route truncations redone by the stack route */
   int64_t factor_live_bytes; /* bytes of the factor at its live ranks: dense words plus
                                 (rows + cols) x rank per admissible block; what one
                                 triangular-solve pass (L then U) reads            */

@@ -763,12 +763,111 @@ __device__ void task_rowmv(Ctx<T>& c, const Task& t, char* smem) {
   }
 }
 
+// ---------------------------------------------------------------- sums of pieces
+constexpr int kStagePieces = 16;
+
+// Chunks of sum_pieces sign X Y^T restricted to the 64 x 64 tile (i0, j0).
+template <class T>
+struct PieceCursor {
+  const Ctx<T>* c;
+  const Piece* pc;
+  const int* w;
+  int nq, i0, j0, q, l0;
+  __device__ bool valid(int qq) const {
+    const Piece& P = pc[qq];
+    return w[qq] > 0 && !(P.pad & PF_DENSE) && max(P.xoff, i0) < min(P.xoff + P.X.rows, i0 + 64) &&
+           max(P.yoff, j0) < min(P.yoff + P.Y.rows, j0 + 64);
+  }
+  __device__ bool seek(int qq) {
+    while (qq < nq && !valid(qq)) ++qq;
+    q = qq;
+    l0 = 0;
+    return q < nq;
+  }
+  __device__ bool first() { return seek(0); }
+  __device__ bool next() {
+    l0 += KC;
+    if (l0 < w[q]) return true;
+    return seek(q + 1);
+  }
+  __device__ Chunk<T> chunk() const {
+    const Piece& P = pc[q];
+    const int xl = max(P.xoff, i0), xh = min(P.xoff + P.X.rows, i0 + 64);
+    const int yl = max(P.yoff, j0), yh = min(P.yoff + P.Y.rows, j0 + 64);
+    const T sg = (P.pad & PF_ALPHA) ? T(P.sign) * T(c->alpha) : T(P.sign);
+    return Chunk<T>{shift(mat(*c, P.X), xl - P.xoff, l0), shift(matT(*c, P.Y), l0, yl - P.yoff), xl - i0, xh - xl,
+                    yh - yl, min(KC, w[q] - l0), yl - j0, sg};
+  }
+};
+
+// acc += the task's pieces restricted to the 64 x 64 tile (i0, j0), staged
+// kStagePieces at a time, all chunks of a stage as one pipeline; returns the
+// flops (thread 0 only).
+template <class T>
+__device__ double pieces_tile(const Ctx<T>& c, const Task& t, int i0, int j0, T (&acc)[4][4], T* As, T* Bs) {
+  __shared__ Piece s_pc[kStagePieces];
+  __shared__ int s_w[kStagePieces];
+  double fl = 0;
+  for (int qb = 0; qb < t.list_count; qb += kStagePieces) {
+    const int nq = min(kStagePieces, t.list_count - qb);
+    __syncthreads();
+    {
+      const int words = nq * (int)(sizeof(Piece) / sizeof(int32_t));
+      const int32_t* src = reinterpret_cast<const int32_t*>(c.pieces + t.list_begin + qb);
+      int32_t* dst = reinterpret_cast<int32_t*>(s_pc);
+      for (int w = threadIdx.x; w < words; w += NT) dst[w] = __ldg(src + w);
+    }
+    __syncthreads();
+    if (threadIdx.x < nq) s_w[threadIdx.x] = ncols(c, s_pc[threadIdx.x].X);
+    __syncthreads();
+    PieceCursor<T> cur{&c, s_pc, s_w, nq, i0, j0, 0, 0};
+    tile_mma_seq(acc, cur, As, Bs, c.tcc);
+    if (threadIdx.x == 0)
+      for (int q = 0; q < nq; ++q)
+        if (cur.valid(q))
+          fl += 2.0 * (min(s_pc[q].xoff + s_pc[q].X.rows, i0 + 64) - max(s_pc[q].xoff, i0)) *
+                (min(s_pc[q].yoff + s_pc[q].Y.rows, j0 + 64) - max(s_pc[q].yoff, j0)) * s_w[q];
+  }
+  return fl;
+}
+
 // ---------------------------------------------------------------- DADD
+// One product, or (TF_PIECES) the sum of the listed pieces added in one pass
+// over c, the window at (a.rows, a.cols) of the target the pieces refer to (an
+// update of a dense block per step and level cost a queue hop and a read and
+// write of c each: 4.7 M tasks at n = 24, now 0.33 M).
 template <class T>
 __device__ void task_dadd(Ctx<T>& c, const Task& t, char* smem) {
-  const int m = t.c.rows, n = ncols(c, t.c), k = ncols(c, t.a);
   T* As = reinterpret_cast<T*>(smem);
   T* Bs = As + kStage;
+  if (t.flags & TF_PIECES) {
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const bool over = (t.flags & TF_OVERWRITE) != 0;
+    double fl = 0;
+    for (int i0 = 0; i0 < t.c.rows; i0 += 64)
+      for (int j0 = 0; j0 < t.c.cols; j0 += 64) {
+        T acc[4][4], base[4][4];
+        acc_zero(acc);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int r = i0 + tx * 4 + i, cc = j0 + ty * 4 + j;
+            base[i][j] = !over && r < t.c.rows && cc < t.c.cols ? ldv(c, t.c, r, cc) : T(0);
+          }
+        fl += pieces_tile(c, t, t.a.rows + i0, t.a.cols + j0, acc, As, Bs);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int r = i0 + tx * 4 + i, cc = j0 + ty * 4 + j;
+            if (r < t.c.rows && cc < t.c.cols) stv(c, t.c, r, cc, base[i][j] + acc[i][j]);
+          }
+      }
+    if (threadIdx.x == 0) c.flops += fl;
+    return;
+  }
+  const int m = t.c.rows, n = ncols(c, t.c), k = ncols(c, t.a);
   for (int i0 = 0; i0 < m; i0 += 64)
     for (int j0 = 0; j0 < n; j0 += 64) {
       T acc[4][4];
@@ -1042,21 +1141,24 @@ __device__ int jacobi_svd(T* G, T* V, int p, int q, T* nrm2, T tol, T negl_rel) 
   for (; sweep < 20 && qq > 1; ++sweep) {
     norms();
     __syncthreads();
-    if (threadIdx.x == 0) {
-      s_rot = 0;
-      s_off = 0.0f;
+    if (threadIdx.x < 32) {
       T mx = 0;
-      for (int j = 0; j < q; ++j) mx = max(mx, nrm2[j]);
-      s_negl = negl_rel * negl_rel * mx;
+      for (int j = lane; j < q; j += 32) mx = max(mx, nrm2[j]);
+      for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      if (lane == 0) {
+        s_rot = 0;
+        s_off = 0.0f;
+        s_negl = negl_rel * negl_rel * mx;
+      }
     }
     __syncthreads();
     for (int rd = 0; rd < qq - 1; ++rd) {
       int a = 0, b = 0;
       bool act = k < npairs;
       if (act) {
-        const int pa = k == 0 ? 0 : ((k - 1 + rd) % (qq - 1)) + 1;
-        const int kb = qq - 1 - k;
-        const int pb = kb == 0 ? 0 : ((kb - 1 + rd) % (qq - 1)) + 1;
+        const int ia = k - 1 + rd, ib = qq - 2 - k + rd;  // round-robin places, modulo qq - 1
+        const int pa = k == 0 ? 0 : (ia >= qq - 1 ? ia - (qq - 1) : ia) + 1;
+        const int pb = (ib >= qq - 1 ? ib - (qq - 1) : ib) + 1;  // qq - 1 - k >= 1 for every pair
         a = min(pa, pb);
         b = max(pa, pb);
         act = b < q;
@@ -1109,8 +1211,8 @@ __device__ int jacobi_svd(T* G, T* V, int p, int q, T* nrm2, T tol, T negl_rel) 
 }
 
 constexpr int kDenseMax = 128;
-constexpr int kDenseRank = 40;           // rows kept by the dense route's pivoted QR
-constexpr int kCoreRank = kRankMax;      // rows kept by the stack route's pivoted QR of the core
+constexpr int kDenseRank = 40;           // columns kept by the dense route
+constexpr int kCoreRank = kRankMax;      // columns kept of the stack route's core
 constexpr int kCoreV = kTruncStack * kCoreRank + kCoreRank * kCoreRank;  // M (q x r') and V (r' x r')
 
 // dynamic shared memory of the task bodies: max over task kinds of TRUNC
@@ -1118,11 +1220,11 @@ constexpr int kCoreV = kTruncStack * kCoreRank + kCoreRank * kCoreRank;  // M (q
 // GEMM chunks (2 x KC x kLds) with a ROWMV's output tile
 __host__ __device__ constexpr size_t exec_smem_base(int elem_size) {
   const size_t trunc0 = (size_t)elem_size * (3 * kTruncStack + kTruncStack * kTruncStack + kCoreV);
-  // dense truncation route (FP32 only)
-  const size_t r0 = (size_t)4 * (kDenseMax * kDenseRank + kDenseRank * kDenseRank);
-  const size_t region0 = r0 < (size_t)4 * 2 * kStage ? (size_t)4 * 2 * kStage : r0;
-  const size_t dense = region0 + (size_t)4 * (kDenseMax * kDenseMax + 2 * kDenseMax) + sizeof(int) * kDenseMax;
-  const size_t trunc = (elem_size == 4 && dense > trunc0) ? dense : trunc0;
+  // dense truncation route
+  const size_t r0 = (size_t)elem_size * (kDenseMax * kDenseRank + kDenseRank * kDenseRank);
+  const size_t region0 = r0 < (size_t)elem_size * 2 * kStage ? (size_t)elem_size * 2 * kStage : r0;
+  const size_t dense = region0 + (size_t)elem_size * (kDenseMax * kDenseMax + 2 * kDenseMax) + sizeof(int) * kDenseMax;
+  const size_t trunc = dense > trunc0 ? dense : trunc0;
   const size_t lu0 = (size_t)elem_size * (64 * 64 + 64) + 64 * sizeof(int);
   const size_t gemm = (size_t)elem_size * (2 * kStage + 64 * 64);
   const size_t m = trunc > lu0 ? trunc : lu0;
@@ -1132,95 +1234,190 @@ __host__ __device__ constexpr size_t exec_smem_base(int elem_size) {
 __host__ __device__ constexpr size_t exec_stage_offset() { return (exec_smem_base(4) + 1023) & ~(size_t)1023; }
 
 
-// Householder QR with column pivoting of D (m x n, ld m, shared memory) in
-// place, stopped after kmax steps or once the trailing block's squared
-// Frobenius norm is <= rel2 ||D||_F^2.  perm[j] = original index of column j.
-// Returns the number of reflectors r'; *tail2 receives the dropped norm^2.
+// Rank-revealing factorisation D ~ Q R of a small matrix (m x n, both at most
+// kDenseMax, ld m, shared memory): modified Gram-Schmidt with column pivoting,
+// stopped after kmax steps or once the remaining columns' squared Frobenius
+// norm is <= rel2 ||D||_F^2.  Step k takes the column of largest norm, perm[k];
+// column perm[k] of D is left as q_k / inv[k], and M (n x kmax, ld n) receives
+// R^T: M[j + k n] = q_k . D_j at that step.  D - Q R is at rounding level
+// whatever the pivots' range (each step subtracts what it records); the
+// q_k of small pivots lose orthogonality only by an amount that is at rounding
+// level of D again once multiplied by their pivot.
+// A warp owns every eighth column and holds eight of them in registers: one
+// pass over D per step computes the products, the update and the new norms
+// (recomputed, not downdated, so the stop is sharp), and one barrier per step
+// suffices because every warp repeats the pivot search on the norms of the
+// step before.  The Householder version took two passes, five barriers and a
+// serial scan of the norms per step (a 128 x 128 truncation 160 us on average at n = 24; now 94 us, two thirds of it the sum and the Jacobi rounds).
+// Returns the number of steps; *tail2 receives the dropped norm^2, *piv2 the
+// first pivot's.
 template <class T>
-__device__ int pivoted_qr(T* D, int m, int n, int kmax, T rel2, T* tau, T* nrm2, int* perm, T* tail2) {
-  __shared__ int s_piv;
-  __shared__ T s_tail, s_thr, s_beta, s_sc, s_tau;
+__device__ int mgs_pivoted(T* D, int m, int n, int kmax, T rel2, T* inv, int* perm, T* M, T* tail2, T* piv2) {
+  __shared__ T s_n2[2][128];
+  constexpr int CG = 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int j = threadIdx.x; j < n; j += NT) perm[j] = j;
   const int kend = min(kmax, min(m, n));
+  T thr = 0, tail = 0;
+  // sums of eight columns over the lanes: lane 4 u ends with column u's
+  auto lane_sums = [&](T(&v)[CG]) {
+#pragma unroll
+    for (int w = 4, o = 16; w > 0; w >>= 1, o >>= 1) {
+      const bool hi = (lane & o) != 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q < w) {
+          const T keep = hi ? v[q + w] : v[q], send = hi ? v[q] : v[q + w];
+          v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return v[0];
+  };
+  for (int g = 0; g < 128 / (CG * (NT / 32)); ++g) {
+    T v[CG];
+#pragma unroll
+    for (int u = 0; u < CG; ++u) {
+      const int c = warp + NT / 32 * (g * CG + u);
+      v[u] = 0;
+      if (c < n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = lane + 32 * i;
+          const T x = r < m ? D[r + c * m] : T(0);
+          v[u] += x * x;
+        }
+    }
+    const T sum = lane_sums(v);
+    const int c = warp + NT / 32 * (g * CG + (lane >> 2));
+    if ((lane & 3) == 0 && c < n) s_n2[0][c] = sum;
+  }
+  __syncthreads();
   int k = 0;
   for (;; ++k) {
-    for (int j = k + warp; j < n; j += NT / 32) {
-      T acc = 0;
-      for (int i = k + lane; i < m; i += 32) acc += D[i + j * m] * D[i + j * m];
-      acc = warp_sum(acc);
-      if (lane == 0) nrm2[j] = acc;
+    const T* n2 = s_n2[k & 1];
+    T* n2w = s_n2[(k + 1) & 1];
+    T best = T(-1);
+    int bi = n;
+    tail = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int c = lane + 32 * i;
+      const T v = c < n ? n2[c] : T(-1);
+      if (v >= T(0)) tail += v;
+      if (v > best) {
+        best = v;
+        bi = c;
+      }
     }
-    __syncthreads();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      tail += __shfl_xor_sync(0xffffffffu, tail, o);
+      const T ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ob > best || (ob == best && oi < bi)) {
+        best = ob;
+        bi = oi;
+      }
+    }
+    if (k == 0) {
+      thr = rel2 * tail;
+      *piv2 = best;
+    }
+    // a norm that is not a number never compares as the largest: the steps end
+    if (k >= kend || tail <= thr || !(best > T(0))) break;
+    const T nrm = sqrt(best), iv = T(1) / nrm;
+    T q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = lane + 32 * i;
+      q[i] = r < m ? D[r + bi * m] * iv : T(0);
+    }
     if (threadIdx.x == 0) {
-      T tail = 0, best = T(-1);
-      int piv = k;
-      for (int j = k; j < n; ++j) {
-        tail += nrm2[j];
-        if (nrm2[j] > best) {
-          best = nrm2[j];
-          piv = j;
+      perm[k] = bi;
+      inv[k] = iv;
+    }
+    for (int g = 0; g < 128 / (CG * (NT / 32)); ++g) {
+      if (warp + NT / 32 * g * CG >= n) break;
+      T x[CG][4], d[CG];
+      bool act[CG];
+#pragma unroll
+      for (int u = 0; u < CG; ++u) {
+        const int c = warp + NT / 32 * (g * CG + u);
+        act[u] = c < n && c != bi && n2[c < n ? c : 0] >= T(0);
+        d[u] = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = lane + 32 * i;
+          x[u][i] = act[u] && r < m ? D[r + c * m] : T(0);
+          d[u] += q[i] * x[u][i];
         }
       }
-      if (k == 0) s_thr = rel2 * tail;
-      s_tail = tail;
-      s_piv = piv;
-    }
-    __syncthreads();
-    if (k >= kend || s_tail <= s_thr) break;
-    const int pv = s_piv;
-    if (pv != k) {
-      for (int i = threadIdx.x; i < m; i += NT) {
-        const T x = D[i + k * m];
-        D[i + k * m] = D[i + pv * m];
-        D[i + pv * m] = x;
-      }
-      if (threadIdx.x == 0) {
-        const int pp = perm[k];
-        perm[k] = perm[pv];
-        perm[pv] = pp;
-      }
-    }
-    __syncthreads();
-    if (warp == 0) {
-      T ss = 0;
-      for (int i = k + 1 + lane; i < m; i += 32) ss += D[i + k * m] * D[i + k * m];
-      ss = warp_sum(ss);
-      if (lane == 0) {
-        const T alpha = D[k + k * m];
-        T beta = alpha, sc = 0, tj = 0;
-        if (ss > T(0)) {
-          const T nrm = sqrt(alpha * alpha + ss);
-          beta = alpha >= T(0) ? -nrm : nrm;
-          sc = T(1) / (alpha - beta);
-          tj = (beta - alpha) / beta;
+      const T dl = lane_sums(d);
+      T v[CG];
+#pragma unroll
+      for (int u = 0; u < CG; ++u) {
+        const T du = __shfl_sync(0xffffffffu, dl, 4 * u);
+        const int c = warp + NT / 32 * (g * CG + u);
+        v[u] = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = lane + 32 * i;
+          x[u][i] -= du * q[i];
+          v[u] += x[u][i] * x[u][i];
+          if (act[u] && r < m) D[r + c * m] = x[u][i];
         }
-        s_beta = beta;
-        s_sc = sc;
-        s_tau = tj;
-        tau[k] = tj;
       }
-      __syncwarp();
-      const T sc = s_sc;
-      for (int i = k + 1 + lane; i < m; i += 32) D[i + k * m] *= sc;
-      __syncwarp();
-      if (lane == 0) D[k + k * m] = s_beta;
+      const T sum = lane_sums(v);
+      const int u = lane >> 2, c = warp + NT / 32 * (g * CG + u);
+      if ((lane & 3) == 0 && c < n) {
+        const bool a = c != bi && n2[c] >= T(0);
+        n2w[c] = a ? sum : T(-1);
+        M[c + k * n] = a ? dl : (c == bi ? nrm : T(0));
+      }
     }
-    __syncthreads();
-    const T tj = s_tau;
-    if (tj != T(0))
-      for (int j = k + 1 + warp; j < n; j += NT / 32) {
-        T d = 0;
-        for (int i = k + 1 + lane; i < m; i += 32) d += D[i + k * m] * D[i + j * m];
-        d = (warp_sum(d) + D[k + j * m]) * tj;
-        for (int i = k + 1 + lane; i < m; i += 32) D[i + j * m] -= d * D[i + k * m];
-        __syncwarp();
-        if (lane == 0) D[k + j * m] -= d;
-      }
     __syncthreads();
   }
-  *tail2 = s_tail;
+  *tail2 = tail;
   return k;
+}
+
+// Z (m x r, ld) <- Q V_sel S: the kept left vectors from mgs_pivoted's columns
+// and the rotations Vs (rp x rp) of the kept columns ord, scaled by sv.
+template <class T, class Put>
+__device__ void mgs_left(const T* D, int m, int rp, int r, const T* inv, const int* perm, const T* Vs, const T* sv,
+                         const int* ord, const Put& put) {
+  for (int e = threadIdx.x; e < m * r; e += NT) {
+    const int i = e % m, j = e / m;
+    const T* v = Vs + ord[j] * rp;
+    T sum = 0;
+    for (int l = 0; l < rp; ++l) sum += D[i + perm[l] * m] * (inv[l] * v[l]);
+    put(i, j, sum * sv[ord[j]]);
+  }
+}
+
+// Singular values sv[j] = sqrt(sv[j]) of the rp columns on the way in, their
+// descending order in ord (equal ones by index), and the number kept:
+// s_i > eps s_1.  Every thread finds one value's place by counting; a NaN
+// counts as smallest and is never kept.
+template <class T>
+__device__ int select_rank(T* sv, int rp, int* ord, double eps, T* smax_out) {
+  const int j = threadIdx.x;
+  T s = j < rp ? sqrt(sv[j]) : T(0);
+  if (!(s >= T(0))) s = T(0);
+  __syncthreads();
+  if (j < rp) sv[j] = s;
+  __syncthreads();
+  T smax = 0;
+  int pos = 0;
+  for (int i = 0; i < rp; ++i) {
+    const T x = sv[i];
+    smax = max(smax, x);
+    pos += x > s || (x == s && i < j);
+  }
+  if (j < rp) ord[pos] = j;
+  *smax_out = smax;
+  return __syncthreads_count(j < rp && s > T(eps) * smax);
 }
 
 // stack width at which a truncation compresses before adding the next piece
@@ -1251,7 +1448,6 @@ __device__ int compress_core(TC* SX, TC* SY, int m, int n, int W, int cap, doubl
       t0 = t1;
     }
   };
-  __shared__ int s_r;
   __shared__ int s_ord[kStackCols];
   __shared__ double s_fro;
   constexpr int kHalf = NT / 2;
@@ -1271,21 +1467,17 @@ __device__ int compress_core(TC* SX, TC* SY, int m, int n, int W, int cap, doubl
   }
   __syncthreads();
   lap(2);
-  // pivoted QR of the core down to the truncation floor (G ~ Q_G R' P^T with
-  // r' rows kept), then the Jacobi SVD of M = P R'^T (q x r'): M V_M = W,
+  // rank-revealing factorisation of the core down to the truncation floor
+  // (G ~ Q_G M^T, M q x r'), then the Jacobi SVD of M: M V_M = W,
   // G ~ Q_G V_M W^T; X <- Q_x Q_G V_M S and Y <- Q_y W S^-1 below
-  __shared__ TC s_tauG[kStackCols];
+  __shared__ TC s_inv[kStackCols];
   __shared__ int s_perm[kStackCols];
-  TC tail2 = 0;
+  TC tail2 = 0, piv2 = 0;
   const TC rel = TC(0.1 * eps);
-  const int rp = pivoted_qr(G, p, q, min(kCoreRank, min(p, q)), rel * rel / TC(min(p, q)), s_tauG, sv, s_perm,
-                            &tail2);
   TC* M = V;
+  const int rp = mgs_pivoted(G, p, q, min(kCoreRank, min(p, q)), rel * rel / TC(min(p, q)), s_inv, s_perm, M, &tail2,
+                             &piv2);
   TC* Vs = V + q * rp;
-  for (int idx = threadIdx.x; idx < q * rp; idx += NT) {
-    const int j = idx % q, i = idx / q;
-    M[s_perm[j] + i * q] = j >= i ? G[i + j * p] : TC(0);
-  }
   for (int idx = threadIdx.x; idx < rp * rp; idx += NT) Vs[idx] = (idx % rp == idx / rp) ? TC(1) : TC(0);
   __syncthreads();
   const int sweeps = rp > 0 ? jacobi_svd(M, Vs, q, rp, sv, TC(jtol), TC(0.01 * eps)) : 0;
@@ -1295,49 +1487,28 @@ __device__ int compress_core(TC* SX, TC* SY, int m, int n, int W, int cap, doubl
     tp[6] += (unsigned long long)sweeps;
     tp[7] += (unsigned long long)W;
   }
+  TC smax = 0;
+  const int want = select_rank(sv, rp, s_ord, eps, &smax);
+  const bool more = rp == kCoreRank && tail2 > TC(eps * eps) * smax * smax;
+  const int r = min(want, cap);
   if (threadIdx.x == 0) {
     double f2 = 0;
-    for (int j = 0; j < rp; ++j) {
-      sv[j] = sqrt(sv[j]);
-      s_ord[j] = j;
-      f2 += (double)sv[j] * (double)sv[j];
-    }
+    for (int j = 0; j < rp; ++j) f2 += (double)sv[j] * (double)sv[j];
     s_fro = sqrt(f2);
-    for (int j = 1; j < rp; ++j) {  // stable insertion sort, descending
-      int x = s_ord[j], i = j - 1;
-      while (i >= 0 && sv[s_ord[i]] < sv[x]) {
-        s_ord[i + 1] = s_ord[i];
-        --i;
-      }
-      s_ord[i + 1] = x;
-    }
-    TC smax = rp ? sv[s_ord[0]] : TC(0);
-    int r = 0;
-    if (smax > TC(0))
-      while (r < rp && sv[s_ord[r]] > TC(eps) * smax) ++r;
-    const bool more = rp == kCoreRank && tail2 > TC(eps * eps) * smax * smax;
-    atomicMax(status + 4, more ? kCoreRank + 1 : r);
-    if (r > cap || more) {
-      r = min(r, cap);
-      atomicAdd(status + 2, 1);
-    }
-    s_r = r;
+    atomicMax(status + 4, more ? kCoreRank + 1 : want);
+    if (want > cap || more) atomicAdd(status + 2, 1);
     *flops += 2.0 * (m + n) * W * W + 4.0 * (double)p * q * rp + 6.0 * sweeps * (double)q * rp * rp +
               2.0 * (m + n) * W * r;
   }
   __syncthreads();
-  const int r = s_r;
   *fro = s_fro;
-  for (int64_t idx = threadIdx.x; idx < (int64_t)m * r; idx += NT) {
-    const int i = (int)(idx % m), j = (int)(idx / m);
-    OX[i + (int64_t)j * ox] = i < rp ? Vs[i + s_ord[j] * rp] * sv[s_ord[j]] : TC(0);
-  }
+  mgs_left(G, p, rp, r, s_inv, s_perm, Vs, sv, s_ord, [&](int i, int j, TC v) { OX[i + (int64_t)j * ox] = v; });
+  for (int64_t idx = threadIdx.x; idx < (int64_t)(m - p) * r; idx += NT)
+    OX[p + idx % (m - p) + idx / (m - p) * ox] = TC(0);
   for (int64_t idx = threadIdx.x; idx < (int64_t)n * r; idx += NT) {
     const int i = (int)(idx % n), j = (int)(idx / n);
     OY[i + (int64_t)j * oy] = i < q ? M[i + s_ord[j] * q] / sv[s_ord[j]] : TC(0);
   }
-  __syncthreads();
-  apply_q_group<TC, NT / 32>(G, p, rp, s_tauG, OX, ox, r, threadIdx.x);
   __syncthreads();
   if (threadIdx.x < kHalf)
     apply_q_group<TC, kHalf / 32>(SX, m, p, tauX, OX, ox, r, threadIdx.x);
@@ -1441,51 +1612,14 @@ __device__ int trunc_stack(Ctx<T>& c, const Task& t, TC* SX, TC* SY, TC* OX, TC*
 }
 
 // ------------------------------------------------------------- dense TRUNC
-// Targets with both sides up to kDenseMax whose pieces would need more than
-// one compression of the stack take a dense route (FP32 factors): the sum
-// D = sum sign X Y^T is formed in shared memory, a Householder QR with column
-// pivoting stops once the trailing block's Frobenius norm is below
+// Targets with both sides up to kDenseMax take a dense route: the sum
+// D = sum sign X Y^T is formed in shared memory, a pivoted Gram-Schmidt stops
+// once the remaining block's Frobenius norm is below
 // 0.1 eps ||D||_F / sqrt(min(m, n)) (<= 0.1 eps s_1), and the one-sided Jacobi
-// SVD of the remaining r' x n rows gives the truncation s_i > eps s_1.
-constexpr int kStagePieces = 16;
-
-// Chunks of sum_pieces sign X Y^T restricted to the 64 x 64 tile (i0, j0).
-template <class T>
-struct PieceCursor {
-  const Ctx<T>* c;
-  const Piece* pc;
-  const int* w;
-  int nq, i0, j0, q, l0;
-  __device__ bool valid(int qq) const {
-    const Piece& P = pc[qq];
-    return w[qq] > 0 && max(P.xoff, i0) < min(P.xoff + P.X.rows, i0 + 64) &&
-           max(P.yoff, j0) < min(P.yoff + P.Y.rows, j0 + 64);
-  }
-  __device__ bool seek(int qq) {
-    while (qq < nq && !valid(qq)) ++qq;
-    q = qq;
-    l0 = 0;
-    return q < nq;
-  }
-  __device__ bool first() { return seek(0); }
-  __device__ bool next() {
-    l0 += KC;
-    if (l0 < w[q]) return true;
-    return seek(q + 1);
-  }
-  __device__ Chunk<T> chunk() const {
-    const Piece& P = pc[q];
-    const int xl = max(P.xoff, i0), xh = min(P.xoff + P.X.rows, i0 + 64);
-    const int yl = max(P.yoff, j0), yh = min(P.yoff + P.Y.rows, j0 + 64);
-    const T sg = (P.pad & PF_ALPHA) ? T(P.sign) * T(c->alpha) : T(P.sign);
-    return Chunk<T>{shift(mat(*c, P.X), xl - P.xoff, l0), shift(matT(*c, P.Y), l0, yl - P.yoff), xl - i0, xh - xl,
-                    yh - yl, min(KC, w[q] - l0), yl - j0, sg};
-  }
-};
-
-// Returns false, having written nothing but the shared memory, when the
-// pivoted QR reached kDenseRank rows with a dropped tail above
-// eps |R_00| (|R_00| <= s_1): the stack route then truncates the target.
+// SVD of its n x r' factor gives the truncation s_i > eps s_1.
+// Returns false, having written nothing but the shared memory, when
+// kDenseRank steps left a tail above eps times the first pivot (<= s_1): the
+// stack route then truncates the target.
 template <class T>
 __device__ bool task_trunc_dense(Ctx<T>& c, const Task& t, char* smem) {
   const int m = t.a.rows, n = t.b.rows;
@@ -1499,39 +1633,29 @@ __device__ bool task_trunc_dense(Ctx<T>& c, const Task& t, char* smem) {
   T* tau = D + kDenseMax * kDenseMax;
   T* nrm2 = tau + kDenseMax;
   int* perm = reinterpret_cast<int*>(nrm2 + kDenseMax);
-  __shared__ Piece s_pc[kStagePieces];
-  __shared__ int s_w[kStagePieces];
   __shared__ int s_ord[kDenseRank];
-  __shared__ int s_r;
   unsigned long long* tp = c.tprof;
   long long t0 = tp && threadIdx.x == 0 ? clock64() : 0;
-  // D = sum of the pieces, tile by tile, pieces staged kStagePieces at a time
+  // D = sum of the pieces, tile by tile (a PF_DENSE piece is its X)
+  __shared__ int s_dense;
+  if (threadIdx.x == 0) s_dense = -1;
+  __syncthreads();
+  for (int q = threadIdx.x; q < t.list_count; q += NT)
+    if (c.pieces[t.list_begin + q].pad & PF_DENSE) s_dense = t.list_begin + q;
+  __syncthreads();
+  const int dense = s_dense;
   for (int i0 = 0; i0 < m; i0 += 64)
     for (int j0 = 0; j0 < n; j0 += 64) {
       T acc[4][4];
       acc_zero(acc);
-      for (int qb = 0; qb < t.list_count; qb += kStagePieces) {
-        const int nq = min(kStagePieces, t.list_count - qb);
-        __syncthreads();
-        {
-          const int words = nq * (int)(sizeof(Piece) / sizeof(int32_t));
-          const int32_t* src = reinterpret_cast<const int32_t*>(c.pieces + t.list_begin + qb);
-          int32_t* dst = reinterpret_cast<int32_t*>(s_pc);
-          for (int w = threadIdx.x; w < words; w += NT) dst[w] = __ldg(src + w);
-        }
-        __syncthreads();
-        if (threadIdx.x < nq) s_w[threadIdx.x] = ncols(c, s_pc[threadIdx.x].X);
-        __syncthreads();
-        PieceCursor<T> cur{&c, s_pc, s_w, nq, i0, j0, 0, 0};
-        tile_mma_seq(acc, cur, As, Bs, c.tcc);
-      }
+      pieces_tile(c, t, i0, j0, acc, As, Bs);
       const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int r = i0 + tx * 4 + i, cc = j0 + ty * 4 + j;
-          if (r < m && cc < n) D[r + cc * m] = acc[i][j];
+          if (r < m && cc < n) D[r + cc * m] = acc[i][j] + (dense >= 0 ? ldv(c, c.pieces[dense].X, r, cc) : T(0));
         }
     }
   __syncthreads();
@@ -1540,25 +1664,21 @@ __device__ bool task_trunc_dense(Ctx<T>& c, const Task& t, char* smem) {
     tp[0] += (unsigned long long)(t1 - t0);
     t0 = t1;
   }
-  // pivoted QR down to the truncation floor
+  // down to the truncation floor: D ~ Q M^T, M n x r'
   const T rel = T(0.1 * c.eps);
-  T tail2 = 0;
-  const int rp = pivoted_qr(D, m, n, kDenseRank, rel * rel / T(min(m, n)), tau, nrm2, perm, &tail2);
+  T tail2 = 0, piv2 = 0;
+  const int rp = mgs_pivoted(D, m, n, kDenseRank, rel * rel / T(min(m, n)), tau, perm, M, &tail2, &piv2);
   if (tp && threadIdx.x == 0) {
     const long long t1 = clock64();
     tp[1] += (unsigned long long)(t1 - t0);
     t0 = t1;
   }
-  if (rp == kDenseRank && tail2 > T(c.eps * c.eps) * D[0] * D[0]) {
+  if (rp == kDenseRank && tail2 > T(c.eps * c.eps) * piv2) {
     if (threadIdx.x == 0) atomicAdd(c.status + 5, 1);
     __syncthreads();
     return false;
   }
-  // M = P R'^T (n x r'), Jacobi SVD of its columns: M V = W
-  for (int idx = threadIdx.x; idx < n * rp; idx += NT) {
-    const int j = idx % n, i = idx / n;
-    M[perm[j] + i * n] = j >= i ? D[i + j * m] : T(0);
-  }
+  // Jacobi SVD of M's columns: M V = W
   for (int idx = threadIdx.x; idx < rp * rp; idx += NT) V[idx] = (idx % rp == idx / rp) ? T(1) : T(0);
   __syncthreads();
   int sweeps = 0;
@@ -1571,43 +1691,16 @@ __device__ bool task_trunc_dense(Ctx<T>& c, const Task& t, char* smem) {
     tp[7] += (unsigned long long)rp;
     t0 = t1;
   }
+  T smax = 0;
+  const int want = select_rank(nrm2, rp, s_ord, c.eps, &smax);
+  const int r = min(want, t.cap);
   if (threadIdx.x == 0) {
-    for (int j = 0; j < rp; ++j) {
-      nrm2[j] = sqrt(nrm2[j]);
-      s_ord[j] = j;
-    }
-    for (int j = 1; j < rp; ++j) {  // stable insertion sort, descending
-      int x = s_ord[j], i = j - 1;
-      while (i >= 0 && nrm2[s_ord[i]] < nrm2[x]) {
-        s_ord[i + 1] = s_ord[i];
-        --i;
-      }
-      s_ord[i + 1] = x;
-    }
-    const T smax = rp ? nrm2[s_ord[0]] : T(0);
-    int r = 0;
-    if (smax > T(0))
-      while (r < rp && nrm2[s_ord[r]] > T(c.eps) * smax) ++r;
-    atomicMax(c.status + 4, r);
-    if (r > t.cap) {
-      r = min(r, t.cap);
-      atomicAdd(c.status + 2, 1);
-    }
-    s_r = r;
-    c.flops += 2.0 * (double)m * n * kDenseRank + 2.0 * (double)m * n * rp + 6.0 * sweeps * (double)n * rp * rp;
+    atomicMax(c.status + 4, want);
+    if (want > t.cap) atomicAdd(c.status + 2, 1);
+    c.flops += 4.0 * (double)m * n * rp + 6.0 * sweeps * (double)n * rp * rp;
   }
-  __syncthreads();
-  const int r = s_r;
-  // X = Q' [V_sel S; 0] through the scratch, Y = W_sel / s
-  T* OX = c.scratch;
-  for (int64_t idx = threadIdx.x; idx < (int64_t)m * r; idx += NT) {
-    const int i = (int)(idx % m), j = (int)(idx / m);
-    OX[i + (int64_t)j * m] = i < rp ? V[i + s_ord[j] * rp] * nrm2[s_ord[j]] : T(0);
-  }
-  __syncthreads();
-  apply_q_group<T, NT / 32>(D, m, rp, tau, OX, m, r, threadIdx.x);
-  __syncthreads();
-  for (int64_t idx = threadIdx.x; idx < (int64_t)m * r; idx += NT) stv(c, t.a, idx % m, idx / m, OX[idx]);
+  // X = Q V_sel S, Y = W_sel / s
+  mgs_left(D, m, rp, r, tau, perm, V, nrm2, s_ord, [&](int i, int j, T v) { stv(c, t.a, i, j, v); });
   for (int64_t idx = threadIdx.x; idx < (int64_t)n * r; idx += NT) {
     const int i = (int)(idx % n), j = (int)(idx / n);
     stv(c, t.b, i, j, M[i + s_ord[j] * n] / nrm2[s_ord[j]]);
@@ -1693,7 +1786,6 @@ __device__ void task_trunc_small(Ctx<T>& c, const Task& t, char* smem, int W) {
   T* Zy = Zx + W * W;
   int* perm = reinterpret_cast<int*>(Zy + W * W);
   int* ord = perm + W;
-  __shared__ int s_r;
   for (int idx = threadIdx.x; idx < (m + n) * W; idx += NT) SX[idx] = T(0);
   __syncthreads();
   int w0 = 0;
@@ -1749,15 +1841,11 @@ __device__ void task_trunc_small(Ctx<T>& c, const Task& t, char* smem, int W) {
   }
   __syncthreads();
   lap(2);
-  T tail2 = 0;
+  T tail2 = 0, piv2 = 0;
   const T rel = T(0.1 * c.eps);
-  const int rp = pivoted_qr(G, p, q, min(kCoreRank, min(p, q)), rel * rel / T(min(p, q)), tauG, sv, perm, &tail2);
   T* M = V;
+  const int rp = mgs_pivoted(G, p, q, min(kCoreRank, min(p, q)), rel * rel / T(min(p, q)), tauG, perm, M, &tail2, &piv2);
   T* Vs = V + q * rp;
-  for (int idx = threadIdx.x; idx < q * rp; idx += NT) {
-    const int j = idx % q, i = idx / q;
-    M[perm[j] + i * q] = j >= i ? G[i + j * p] : T(0);
-  }
   for (int idx = threadIdx.x; idx < rp * rp; idx += NT) Vs[idx] = (idx % rp == idx / rp) ? T(1) : T(0);
   __syncthreads();
   const int sweeps = rp > 0 ? jacobi_svd(M, Vs, q, rp, sv, T(c.jacobi_tol), T(0.01 * c.eps)) : 0;
@@ -1767,46 +1855,23 @@ __device__ void task_trunc_small(Ctx<T>& c, const Task& t, char* smem, int W) {
     tp[6] += (unsigned long long)sweeps;
     tp[7] += (unsigned long long)W;
   }
+  T smax = 0;
+  const int want = select_rank(sv, rp, ord, c.eps, &smax);
+  const bool more = rp == kCoreRank && tail2 > T(c.eps * c.eps) * smax * smax;
+  const int r = min(want, t.cap);
   if (threadIdx.x == 0) {
-    for (int j = 0; j < rp; ++j) {
-      sv[j] = sqrt(sv[j]);
-      ord[j] = j;
-    }
-    for (int j = 1; j < rp; ++j) {  // stable insertion sort, descending
-      int x = ord[j], i = j - 1;
-      while (i >= 0 && sv[ord[i]] < sv[x]) {
-        ord[i + 1] = ord[i];
-        --i;
-      }
-      ord[i + 1] = x;
-    }
-    const T smax = rp ? sv[ord[0]] : T(0);
-    int r = 0;
-    if (smax > T(0))
-      while (r < rp && sv[ord[r]] > T(c.eps) * smax) ++r;
-    const bool more = rp == kCoreRank && tail2 > T(c.eps * c.eps) * smax * smax;
-    atomicMax(c.status + 4, more ? kCoreRank + 1 : r);
-    if (r > t.cap || more) {
-      r = min(r, t.cap);
-      atomicAdd(c.status + 2, 1);
-    }
-    s_r = r;
+    atomicMax(c.status + 4, more ? kCoreRank + 1 : want);
+    if (want > t.cap || more) atomicAdd(c.status + 2, 1);
     c.flops += 2.0 * (m + n) * W * W + 4.0 * (double)p * q * rp + 6.0 * sweeps * (double)q * rp * rp +
                2.0 * (m + n) * W * r;
   }
-  __syncthreads();
-  const int r = s_r;
   // Z_x = Q_G [V_M S; 0] (p x r), Z_y = W S^-1 (q x r), columns by descending s
-  for (int idx = threadIdx.x; idx < p * r; idx += NT) {
-    const int i = idx % p, j = idx / p;
-    Zx[idx] = i < rp ? Vs[i + ord[j] * rp] * sv[ord[j]] : T(0);
-  }
+  mgs_left(G, p, rp, r, tauG, perm, Vs, sv, ord, [&](int i, int j, T v) { Zx[i + j * p] = v; });
   for (int idx = threadIdx.x; idx < q * r; idx += NT) {
     const int i = idx % q, j = idx / q;
     Zy[idx] = M[i + ord[j] * q] / sv[ord[j]];
   }
   __syncthreads();
-  apply_q_group<T, NT / 32>(G, p, rp, tauG, Zx, p, r, threadIdx.x);
   if (threadIdx.x < kHalf)
     orgqr_group<T, kHalf / 32>(SX, m, p, tauX, threadIdx.x, 1);
   else
@@ -1829,6 +1894,581 @@ __device__ void task_trunc_small(Ctx<T>& c, const Task& t, char* smem, int W) {
   if (threadIdx.x == 0) __stcg(c.ranks + t.out_slot, r);
 }
 
+// ---------------------------------------------------------- sampled TRUNC
+// Targets above kDenseMax whose stack is wide: the range of
+// A = sum sign X Y^T is found from k <= 96 random samples (the randomised
+// range finder of Halko, Martinsson and Tropp, "Finding structure with
+// randomness", SIAM Review 53, 2011), so that every pass over the pieces is a
+// 64 x 64-tiled product instead of a column-by-column Householder step:
+//   T = Y^T Omega,  S = X T          (Omega: signs from a hash of the index)
+//   S ~ Q R_S                        (pivoted Gram-Schmidt down to the floor)
+//   U = X^T Q,      M = Y U          (A ~ Q M^T)
+//   M = P R,  R V = W (Jacobi)       X <- Q V S, Y <- P W S^-1, s_i > eps s_1
+// The samples that the pivots leave over estimate what Q misses: their mean
+// square is ||A - Q Q^T A||_F^2, and the first pivot's share of all samples'
+// energy times ||A||_F^2 is at most s_1^2.  The steps stop once the one is
+// below (0.1 eps)^2 of the other.  In FP32, at the end (6 samples left over,
+// or 64 columns kept) (0.55 eps)^2 will do, or eps^2 when the last nine pivots are level: what is missed is then
+// spread over many directions (the rounding of cancelling pieces), each far
+// below the Frobenius norm.  Otherwise, or when a Gram matrix is numerically
+// singular, the task falls back to the stack route (nothing has been written yet).
+// Q and P are orthonormalised once more by their Gram matrices: the
+// Gram-Schmidt vectors of small pivots are only as orthogonal as the pivots' range.
+constexpr int kRsCols = 1024;   // stacked columns
+constexpr int kRsPieces = 64;
+constexpr int kRsMin = 24;      // narrower stacks take the stack routes
+constexpr int kRsSamples = 96;  // of which at most 64 columns are kept
+
+constexpr int kRsStage = 5760;  // staged operands of tile_loop, the largest of its shapes
+
+template <class T>
+struct RsSmem {
+  T st[kRsStage];
+  T E[64 * 64];                 // triangular inverse, later the Jacobi rotations
+  T G[64 * 64];                 // Gram matrix; st, E and G also hold S or M during the Gram-Schmidt
+  T R1[64 * 64];                // (G and R1 stage the last products)
+  T n2[2][kRsSamples], inv[64], sv[64];
+  int perm[64], ord[64];
+  int64_t xb[kRsPieces], yb[kRsPieces];  // arena offset of target row 0 of a piece's column 0
+  int xrs[kRsPieces], xcs[kRsPieces], xlo[kRsPieces], xhi[kRsPieces];
+  int yrs[kRsPieces], ycs[kRsPieces], ylo[kRsPieces], yhi[kRsPieces];
+  T sign[kRsPieces];
+  int pre[kRsPieces + 1];
+  short piece[kRsCols];
+  int fail;
+};
+
+// Shape of a tile product with TX x (256 / TX) threads of 4 x 4 elements: the
+// narrower the result, the taller the tile, so that 16 or 32 kept columns do
+// not pay for 64.
+template <int TX>
+struct TileShape {
+  static constexpr int R = 4 * TX, N = 4 * (NT / TX), K = TX == 64 ? 16 : 32;
+  static constexpr int PA = R + 8, PB = N + 8;
+  static_assert(K * (PA + PB) <= kRsStage, "staged operands");
+};
+// acc += sum over chunks [j0, j1) of A (R x K) B (K x N): fa(kk0 + kk, x) and
+// fb(kk0 + kk, c) give the elements; ac / bc: contiguous along x / c (else
+// along kk, then a warp takes 4 consecutive kk of 8 x).  Registers hold the
+// next chunk while one is multiplied.
+template <int TX, class T, class FA, class FB>
+__device__ __forceinline__ void tile_loop(T (&acc)[4][4], int j0, int j1, bool ac, bool bc, const FA& fa, const FB& fb,
+                                          T* st) {
+  using H = TileShape<TX>;
+  if (j0 >= j1) return;
+  T* As = st;
+  T* Bs = st + H::K * H::PA;
+  constexpr int NA = H::R * H::K / NT, NB = (H::N * H::K + NT - 1) / NT;
+  T ra[NA], rb[NB];
+  auto coord = [](bool cx, int len, int e, int& x, int& kk) {
+    if (cx) {
+      x = e & (len - 1);
+      kk = e / len;
+    } else {
+      kk = ((e >> 5) & (H::K / 4 - 1)) * 4 + (e & 3);
+      x = (e / (8 * H::K)) * 8 + ((e >> 2) & 7);
+    }
+  };
+  auto fetch = [&](int j) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      int x, kk;
+      coord(ac, H::R, threadIdx.x + q * NT, x, kk);
+      ra[q] = fa(j * H::K + kk, x);
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      int x, kk;
+      coord(bc, H::N, threadIdx.x + q * NT, x, kk);
+      rb[q] = fb(j * H::K + kk, x);
+    }
+  };
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  fetch(j0);
+  for (int j = j0; j < j1; ++j) {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      int x, kk;
+      coord(ac, H::R, threadIdx.x + q * NT, x, kk);
+      As[kk * H::PA + x] = ra[q];
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      int x, kk;
+      coord(bc, H::N, threadIdx.x + q * NT, x, kk);
+      Bs[kk * H::PB + x] = rb[q];
+    }
+    __syncthreads();
+    if (j + 1 < j1) fetch(j + 1);
+#pragma unroll 8
+    for (int kk = 0; kk < H::K; ++kk) {
+      T a[4], b[4];
+      lds4(As + kk * H::PA + tx * 4, a);
+      lds4(Bs + kk * H::PB + ty * 4, b);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[i][q] += a[i] * b[q];
+    }
+  }
+  __syncthreads();
+}
+template <int TX, class T, class Put>
+__device__ __forceinline__ void tile_put(const T (&acc)[4][4], int rows, int cols, const Put& put) {
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (tx * 4 + i < rows && ty * 4 + j < cols) put(tx * 4 + i, ty * 4 + j, acc[i][j]);
+}
+// C (rows x cols) tile by tile: element (kk, x) of A from fa, (kk, c) of B from
+// fb, summed over kk < inner
+template <int TX, class T, class FA, class FB, class Put>
+__device__ __forceinline__ void product_tx(int rows, int cols, int inner, bool ac, bool bc, const FA& fa, const FB& fb,
+                                           const Put& put, T* st) {
+  using H = TileShape<TX>;
+  for (int i0 = 0; i0 < rows; i0 += H::R) {
+    T acc[4][4];
+    acc_zero(acc);
+    tile_loop<TX>(
+        acc, 0, (inner + H::K - 1) / H::K, ac, bc, [&](int kk, int x) { return fa(kk, i0 + x); }, fb, st);
+    tile_put<TX>(acc, min(H::R, rows - i0), cols, [&](int i, int j, T v) { put(i0 + i, j, v); });
+  }
+}
+template <class T, class FA, class FB, class Put>
+__device__ __forceinline__ void product(int rows, int cols, int inner, bool ac, bool bc, const FA& fa, const FB& fb,
+                                        const Put& put, T* st) {
+  if (cols <= 16)
+    product_tx<64>(rows, cols, inner, ac, bc, fa, fb, put, st);
+  else if (cols <= 32)
+    product_tx<32>(rows, cols, inner, ac, bc, fa, fb, put, st);
+  else
+    product_tx<16>(rows, cols, inner, ac, bc, fa, fb, put, st);
+}
+
+// Pivoted Gram-Schmidt of S (m x k, ld m, k <= 96, shared memory or global
+// scratch) as mgs_pivoted, for tall columns: a warp holds two columns of up to
+// 512 rows in registers, longer ones take a second pass.  stop(j, tail, first) ends the
+// steps (first: the first pivot's squared norm).  R (64 x 64, ld 64, may be null) receives the coefficients, column by
+// original column.
+template <class T, class Stop>
+__device__ int mgs_tall(T* S, int m, int k, int kmax, RsSmem<T>& sm, T* R, const Stop& stop, T* tail_out, T* first_out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int RL = 16;  // rows of a lane held in registers
+  auto norm_of = [&](int c) {
+    const T* s = S + (int64_t)c * m;
+    T v = 0;
+#pragma unroll 8
+    for (int r = lane; r < m; r += 32) v += s[r] * s[r];
+    return warp_sum(v);
+  };
+  for (int c = warp; c < k; c += NT / 32) {
+    const T v = norm_of(c);
+    if (lane == 0) sm.n2[0][c] = v;
+  }
+  __syncthreads();
+  T first = 0, tail = 0;
+  int j = 0;
+  for (;; ++j) {
+    const T* n2 = sm.n2[j & 1];
+    T* n2w = sm.n2[(j + 1) & 1];
+    T best = T(-1);
+    int bi = k;
+    tail = 0;
+#pragma unroll
+    for (int i = 0; i < kRsSamples / 32; ++i) {
+      const int c = lane + 32 * i;
+      const T v = c < k ? n2[c] : T(-1);
+      if (v >= T(0)) tail += v;
+      if (v > best) {
+        best = v;
+        bi = c;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      tail += __shfl_xor_sync(0xffffffffu, tail, o);
+      const T ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ob > best || (ob == best && oi < bi)) {
+        best = ob;
+        bi = oi;
+      }
+    }
+    if (j == 0) first = best;
+    if (j >= kmax || !(best > T(0)) || stop(j, tail, first)) break;
+    const T nrm = sqrt(best), iv = T(1) / nrm;
+    if (threadIdx.x == 0) {
+      sm.perm[j] = bi;
+      sm.inv[j] = iv;
+    }
+    const T* p = S + (int64_t)bi * m;
+    for (int c0 = warp; c0 < k; c0 += 2 * (NT / 32)) {
+      const int c1 = c0 + NT / 32;
+      const bool a0 = c0 != bi && n2[c0] >= T(0), a1 = c1 < k && c1 != bi && n2[c1 < k ? c1 : 0] >= T(0);
+      T d0 = 0, d1 = 0, v0 = 0, v1 = 0;
+      if (a0 || a1) {
+        T* s0 = S + (int64_t)(a0 ? c0 : c1) * m;
+        T* s1 = S + (int64_t)(a1 ? c1 : c0) * m;
+        if (m <= 32 * RL) {
+          T q[RL], x[RL], y[RL];
+#pragma unroll
+          for (int i = 0; i < RL; ++i) {
+            const int r = lane + 32 * i;
+            q[i] = r < m ? p[r] * iv : T(0);
+            x[i] = r < m ? s0[r] : T(0);
+            y[i] = r < m ? s1[r] : T(0);
+          }
+#pragma unroll
+          for (int i = 0; i < RL; ++i) {
+            d0 += q[i] * x[i];
+            d1 += q[i] * y[i];
+          }
+          d0 = warp_sum(d0);
+          d1 = warp_sum(d1);
+#pragma unroll
+          for (int i = 0; i < RL; ++i) {
+            const int r = lane + 32 * i;
+            x[i] -= d0 * q[i];
+            y[i] -= d1 * q[i];
+            v0 += x[i] * x[i];
+            v1 += y[i] * y[i];
+            if (r < m && a0) s0[r] = x[i];
+            if (r < m && a1) s1[r] = y[i];
+          }
+        } else {
+#pragma unroll 8
+          for (int r = lane; r < m; r += 32) {
+            const T q = p[r] * iv;
+            d0 += q * s0[r];
+            d1 += q * s1[r];
+          }
+          d0 = warp_sum(d0);
+          d1 = warp_sum(d1);
+          for (int r0 = lane; r0 < m; r0 += 32 * 8) {
+            T q[8], x[8], y[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int r = r0 + 32 * i;
+              q[i] = r < m ? p[r] * iv : T(0);
+              x[i] = r < m ? s0[r] : T(0);
+              y[i] = r < m ? s1[r] : T(0);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int r = r0 + 32 * i;
+              x[i] -= d0 * q[i];
+              y[i] -= d1 * q[i];
+              v0 += x[i] * x[i];
+              v1 += y[i] * y[i];
+              if (r < m && a0) s0[r] = x[i];
+              if (r < m && a1) s1[r] = y[i];
+            }
+          }
+        }
+        v0 = warp_sum(v0);
+        v1 = warp_sum(v1);
+      }
+      if (lane == 0) {
+        n2w[c0] = a0 ? v0 : T(-1);
+        if (R) R[j + 64 * c0] = a0 ? d0 : (c0 == bi ? nrm : T(0));
+        if (c1 < k) {
+          n2w[c1] = a1 ? v1 : T(-1);
+          if (R) R[j + 64 * c1] = a1 ? d1 : (c1 == bi ? nrm : T(0));
+        }
+      }
+    }
+    __syncthreads();
+  }
+  *tail_out = tail;
+  *first_out = first;
+  return j;
+}
+
+// Q (m x r, ld m) <- S1 G^-1/2 (Cholesky), S1 (m x r, ld m) the Gram-Schmidt
+// vectors: one more orthonormalisation.  With G = L L^T the elimination of
+// [G | I] leaves L's columns below G's diagonal and D^1/2 L^-1 in E.  Sets
+// sm.fail when a pivot shows S1 numerically dependent.
+template <class T>
+__device__ void gram_orthonormalise(const T* S1, int m, int r, T* Q, RsSmem<T>& sm) {
+  auto at = [&](int row, int x) { return x < r && row < m ? S1[(int64_t)x * m + row] : T(0); };
+  product(
+      r, r, m, false, false, at, at,
+      [&](int i, int j, T v) {
+        sm.G[i + 64 * j] = v;
+        sm.E[i + 64 * j] = i == j ? T(1) : T(0);
+      },
+      sm.st);
+  __syncthreads();
+  for (int j = 0; j < r; ++j) {
+    const T d = sm.G[j + 64 * j];
+    if (!(d > T(0.05))) {
+      if (threadIdx.x == 0) sm.fail = 1;
+      break;
+    }
+    const T dinv = T(1) / d;
+    const int rows = r - 1 - j;
+    for (int e = threadIdx.x; e < rows * r; e += NT) {
+      const int i = j + 1 + e % rows, c = e / rows;
+      const T f = sm.G[i + 64 * j] * dinv;
+      if (c > j)
+        sm.G[i + 64 * c] -= f * sm.G[j + 64 * c];
+      else
+        sm.E[i + 64 * c] -= f * sm.E[j + 64 * c];
+    }
+    __syncthreads();
+  }
+  __syncthreads();
+  if (sm.fail) return;
+  product(
+      m, r, r, true, false,
+      [&](int b, int row) { return b < r && row < m ? S1[(int64_t)b * m + row] : T(0); },
+      [&](int b, int cc) { return b <= cc && cc < r ? sm.E[cc + 64 * b] * rsqrt(sm.G[cc + 64 * cc]) : T(0); },
+      [&](int i, int j, T v) { Q[i + (int64_t)j * m] = v; }, sm.st);
+  __syncthreads();
+}
+
+// Gram-Schmidt of S (global, m x k) through shared memory when it fits there;
+// the chosen columns, normalised, go to S1 (m x steps).
+template <class T, class Stop>
+__device__ int mgs_columns(T* S, int m, int k, int kmax, T* S1, RsSmem<T>& sm, T* R, const Stop& stop, T* tail,
+                           T* first) {
+  constexpr int kFit = kRsStage + 2 * 64 * 64;  // st, E, G
+  T* W = S;
+  if (m * k <= kFit) {
+    W = sm.st;
+    for (int e = threadIdx.x; e < m * k; e += NT) W[e] = S[e];
+    __syncthreads();
+  }
+  const int r = mgs_tall(W, m, k, kmax, sm, R, stop, tail, first);
+  for (int e = threadIdx.x; e < m * r; e += NT) {
+    const int i = e % m, j = e / m;
+    S1[e] = W[(int64_t)sm.perm[j] * m + i] * sm.inv[j];
+  }
+  __syncthreads();
+  return r;
+}
+
+template <class T>
+__device__ bool task_trunc_sampled(Ctx<T>& c, const Task& t, char* smem, int W) {
+  RsSmem<T>& sm = *reinterpret_cast<RsSmem<T>*>(smem);
+  static_assert(sizeof(RsSmem<T>) <= exec_smem_base(sizeof(T)), "the sampled route's shared memory");
+  const int m = t.a.rows, n = t.b.rows, np = t.list_count;
+  const T* arena = c.arena;
+  unsigned long long* tp = c.tprof;
+  long long t0 = tp && threadIdx.x == 0 ? clock64() : 0;
+  auto lap = [&](int k) {
+    if (tp && threadIdx.x == 0) {
+      const long long t1 = clock64();
+      tp[k] += (unsigned long long)(t1 - t0);
+      t0 = t1;
+    }
+  };
+  // the pieces, their column ranges and each column's piece
+  __shared__ int s_wmax;
+  if (threadIdx.x == 0) {
+    sm.fail = 0;
+    s_wmax = 0;
+    sm.pre[0] = 0;
+  }
+  __syncthreads();
+  if (threadIdx.x < np) {
+    const Piece& P = c.pieces[t.list_begin + threadIdx.x];
+    const int p = threadIdx.x;
+    sm.xrs[p] = P.X.rs, sm.xcs[p] = P.X.cs, sm.xlo[p] = P.xoff, sm.xhi[p] = P.xoff + P.X.rows;
+    sm.yrs[p] = P.Y.rs, sm.ycs[p] = P.Y.cs, sm.ylo[p] = P.yoff, sm.yhi[p] = P.yoff + P.Y.rows;
+    sm.xb[p] = P.X.off - (int64_t)P.xoff * P.X.rs;
+    sm.yb[p] = P.Y.off - (int64_t)P.yoff * P.Y.rs;
+    sm.sign[p] = (P.pad & PF_ALPHA) ? T(P.sign) * T(c.alpha) : T(P.sign);
+    const int w = ncols(c, P.X);
+    sm.pre[p + 1] = w;
+    atomicMax(&s_wmax, w);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int p = 0; p < np; ++p) sm.pre[p + 1] += sm.pre[p];
+  __syncthreads();
+  for (int p = threadIdx.x >> 5; p < np; p += NT / 32)
+    for (int q = sm.pre[p] + (threadIdx.x & 31); q < sm.pre[p + 1]; q += 32) sm.piece[q] = (short)p;
+  __syncthreads();
+  // samples: the widest piece's rank and some to spare
+  const int k = s_wmax <= 16 ? 32 : s_wmax <= 32 ? 64 : kRsSamples;
+  T* S = c.scratch;                     // m x 96, later M: n x 64
+  T* S1 = S + c.rows_max * kRsSamples;  // m x 64, later n x 64
+  T* Q = S1 + c.rows_max * 64;          // m x 64
+  T* P = Q + c.rows_max * 64;           // n x 64
+  T* Tm = P + c.rows_max * 64;          // kRsCols x 96
+  // column q of the stacked X (or Y) at target row r
+  auto xat = [&](int q, int r) {
+    if (q >= W || r >= m) return T(0);
+    const int p = sm.piece[q];
+    return r >= sm.xlo[p] && r < sm.xhi[p]
+               ? __ldcg(arena + sm.xb[p] + (int64_t)r * sm.xrs[p] + (int64_t)(q - sm.pre[p]) * sm.xcs[p])
+               : T(0);
+  };
+  auto yat = [&](int q, int r) {
+    if (q >= W || r >= n) return T(0);
+    const int p = sm.piece[q];
+    return r >= sm.ylo[p] && r < sm.yhi[p]
+               ? __ldcg(arena + sm.yb[p] + (int64_t)r * sm.yrs[p] + (int64_t)(q - sm.pre[p]) * sm.ycs[p])
+               : T(0);
+  };
+  // Tm (W x kc) <- sign * stacked^T B, B(row, column) from fb
+  auto project_tx = [&](auto tx, const auto& at, const int* lo, const int* hi, int c0, int kc, const auto& fb) {
+    constexpr int TX = decltype(tx)::value;
+    using H = TileShape<TX>;
+    for (int q0 = 0; q0 < W; q0 += H::R) {
+      int r0 = 1 << 30, r1 = 0;  // rows that the tile's pieces cover
+      for (int p = sm.piece[q0]; p <= sm.piece[min(W, q0 + H::R) - 1]; ++p) {
+        r0 = min(r0, lo[p]);
+        r1 = max(r1, hi[p]);
+      }
+      T acc[4][4];
+      acc_zero(acc);
+      tile_loop<TX>(
+          acc, r0 / H::K, (r1 + H::K - 1) / H::K, false, false, [&](int r, int x) { return at(q0 + x, r); },
+          [&](int r, int cc) { return cc < kc ? fb(r, c0 + cc) : T(0); }, sm.st);
+      tile_put<TX>(acc, min(H::R, W - q0), kc,
+                   [&](int i, int j, T v) { Tm[q0 + i + (c0 + j) * kRsCols] = v * sm.sign[sm.piece[q0 + i]]; });
+    }
+    __syncthreads();
+  };
+  // O (rows x kc, ld rows) <- stacked Tm
+  auto expand_tx = [&](auto tx, const auto& at, const int* lo, const int* hi, int rows, int c0, int kc, T* O) {
+    constexpr int TX = decltype(tx)::value;
+    using H = TileShape<TX>;
+    for (int i0 = 0; i0 < rows; i0 += H::R) {
+      T acc[4][4];
+      acc_zero(acc);
+      auto hit = [&](int q0) {  // whether the chunk's pieces touch these rows
+        bool h = false;
+        for (int p = sm.piece[q0]; p <= sm.piece[min(W, q0 + H::K) - 1]; ++p) h = h || (lo[p] < i0 + H::R && hi[p] > i0);
+        return h;
+      };
+      for (int j0 = 0; j0 < W; j0 += H::K) {
+        if (!hit(j0)) continue;
+        int j1 = j0 + H::K;
+        while (j1 < W && hit(j1)) j1 += H::K;
+        tile_loop<TX>(
+            acc, j0 / H::K, j1 / H::K, true, false, [&](int q, int x) { return at(q, i0 + x); },
+            [&](int q, int cc) { return q < W && cc < kc ? Tm[q + (c0 + cc) * kRsCols] : T(0); }, sm.st);
+        j0 = j1 - H::K;
+      }
+      tile_put<TX>(acc, min(H::R, rows - i0), kc, [&](int i, int j, T v) { O[i0 + i + (int64_t)(c0 + j) * rows] = v; });
+    }
+    __syncthreads();
+  };
+  auto by_width = [&](int kc, const auto& f) {  // f(shape, first column, columns)
+    int c0 = 0;
+    for (; kc - c0 > 32; c0 += 64) f(std::integral_constant<int, 16>(), c0, min(64, kc - c0));
+    if (c0 >= kc) return;
+    if (kc - c0 > 16)
+      f(std::integral_constant<int, 32>(), c0, kc - c0);
+    else
+      f(std::integral_constant<int, 64>(), c0, kc - c0);
+  };
+  auto project = [&](const auto& at, const int* lo, const int* hi, int kc, const auto& fb) {
+    by_width(kc, [&](auto tx, int c0, int w) { project_tx(tx, at, lo, hi, c0, w, fb); });
+  };
+  auto expand = [&](const auto& at, const int* lo, const int* hi, int rows, int kc, T* O) {
+    by_width(kc, [&](auto tx, int c0, int w) { expand_tx(tx, at, lo, hi, rows, c0, w, O); });
+  };
+  // random signs: the finaliser of MurmurHash3 (Appleby) of the index
+  auto omega = [&](int r, int cc) {
+    uint32_t h = (uint32_t)(r * kRsSamples + cc) + 0x9e3779b9u;
+    h ^= h >> 16;
+    h *= 0x85ebca6bu;
+    h ^= h >> 13;
+    h *= 0xc2b2ae35u;
+    h ^= h >> 16;
+    return (h & 1u) ? T(1) : T(-1);
+  };
+  project(yat, sm.ylo, sm.yhi, k, omega);
+  expand(xat, sm.xlo, sm.xhi, m, k, S);
+  lap(0);
+  const T f2 = T(0.01 * c.eps * c.eps);
+  T tail = 0, first = 0;
+  const int kend = min(min(k - 6, 64), min(m, n));
+  const int rp = mgs_columns(
+      S, m, k, kend, S1, sm, (T*)nullptr,
+      [&](int j, T tl, T fst) { return tl * T(k) <= f2 * fst * T(k - j); }, &tail, &first);
+  if (rp == kend) {
+    // (sm.inv holds 1 / pivot norm)
+    const T miss = tail * T(k) / (f2 * first * T(k - rp));  // (missed / 0.1 eps s_1)^2
+    const bool flat = rp >= 16 && sm.inv[rp - 9] >= T(0.5) * sm.inv[rp - 1];
+    if (!(miss <= T(sizeof(T) == 4 ? 30 : 1) || (sizeof(T) == 4 && flat && miss <= T(100)))) {
+      if (threadIdx.x == 0) atomicAdd(c.status + 5, 1);
+      return false;
+    }
+  }
+  if (rp == 0) {
+    __syncthreads();
+    if (threadIdx.x == 0) __stcg(c.ranks + t.out_slot, 0);
+    return true;
+  }
+  gram_orthonormalise(S1, m, rp, Q, sm);
+  if (sm.fail) return false;
+  lap(1);
+  project(xat, sm.xlo, sm.xhi, rp, [&](int r, int cc) { return r < m ? Q[r + (int64_t)cc * m] : T(0); });
+  T* M = S;
+  expand(yat, sm.ylo, sm.yhi, n, rp, M);
+  lap(2);
+  // M = P R: R1 from the Gram-Schmidt, then R = L^T R1
+  T mt = 0, mtot = 0;
+  const int rr = mgs_columns(M, n, rp, rp, S1, sm, sm.R1, [](int, T, T) { return false; }, &mt, &mtot);
+  if (rr == 0) return false;
+  gram_orthonormalise(S1, n, rr, P, sm);
+  if (sm.fail) return false;
+  // the triangular factor: L(i, a) = G(i, a) / sqrt(G(a, a)), i >= a
+  T* R = sm.st;  // rr x rp, ld rr: the staging buffers are free now
+  static_assert(kRsStage >= 64 * 64, "R in the staging buffers");
+  for (int e = threadIdx.x; e < rr * rp; e += NT) {
+    const int a = e % rr, cc = e / rr;
+    T v = 0;
+    for (int i = a; i < rr; ++i) v += sm.G[i + 64 * a] * sm.R1[i + 64 * cc];
+    R[e] = v * rsqrt(sm.G[a + 64 * a]);
+  }
+  __syncthreads();
+  T* V = sm.E;
+  for (int e = threadIdx.x; e < rp * rp; e += NT) V[e] = (e % rp == e / rp) ? T(1) : T(0);
+  __syncthreads();
+  lap(1);
+  const int sweeps = jacobi_svd(R, V, rr, rp, sm.sv, T(c.jacobi_tol), T(0.01 * c.eps));
+  lap(3);
+  if (tp && threadIdx.x == 0) {
+    tp[5] += 1ULL;
+    tp[6] += (unsigned long long)sweeps;
+    tp[7] += (unsigned long long)W;
+  }
+  T smax = 0;
+  const int want = select_rank(sm.sv, rp, sm.ord, c.eps, &smax);
+  const int r = min(want, t.cap);
+  if (threadIdx.x == 0) {
+    atomicMax(c.status + 4, want);
+    if (want > t.cap) atomicAdd(c.status + 2, 1);
+    c.flops += 2.0 * (double)(m + n) * W * (k + rp) + 4.0 * ((double)m * k + (double)n * rp) * rp +
+               6.0 * sweeps * (double)rr * rp * rp + 2.0 * (double)(m + n) * rp * r;
+  }
+  // X = Q V_sel S, Y = P W_sel / s
+  auto put = [&](const T* B, int rows, int inner, const View& out, const auto& z) {
+    product(
+        rows, r, inner, true, false,
+        [&](int b, int row) { return b < inner && row < rows ? B[row + (int64_t)b * rows] : T(0); },
+        [&](int b, int cc) { return b < inner && cc < r ? z(b, cc) : T(0); },
+        [&](int i, int j, T v) { stv(c, out, i, j, v); }, sm.G);
+  };
+  static_assert(2 * 64 * 64 >= kRsStage, "the staged operands in G and R1");
+  __syncthreads();
+  put(Q, m, rp, t.a, [&](int b, int cc) { return V[b + sm.ord[cc] * rp] * sm.sv[sm.ord[cc]]; });
+  put(P, n, rr, t.b, [&](int b, int cc) { return R[b + sm.ord[cc] * rr] / sm.sv[sm.ord[cc]]; });
+  __syncthreads();
+  if (threadIdx.x == 0) __stcg(c.ranks + t.out_slot, r);
+  lap(4);
+  return true;
+}
+
 template <class T>
 __device__ void task_trunc(Ctx<T>& c, const Task& t, char* smem) {
   const int m = t.a.rows, n = t.b.rows;
@@ -1843,13 +2483,17 @@ __device__ void task_trunc(Ctx<T>& c, const Task& t, char* smem) {
   __syncthreads();
   const int wsum = s_wsum;
   __syncthreads();
-  // dense route when the stack would need more than one compression
-  if (sizeof(T) == 4 && m <= kDenseMax && n <= kDenseMax && wsum > c.compress_at && task_trunc_dense(c, t, smem))
-    return;
   if (wsum == 0) {
     if (threadIdx.x == 0) __stcg(c.ranks + t.out_slot, 0);
     return;
   }
+  if (m <= kDenseMax && n <= kDenseMax && task_trunc_dense(c, t, smem)) return;
+  // below kRsEps the floor is under the rounding of the samples
+  constexpr double kRsEps = sizeof(T) == 4 ? 4e-6 : 1e-13;
+  if (wsum > kRsMin && wsum <= kRsCols && t.list_count <= kRsPieces && min(m, n) >= 64 && c.eps >= kRsEps &&
+      task_trunc_sampled(c, t, smem, wsum))
+    return;
+  __syncthreads();
   // the whole stack in shared memory, one compression
   if (trunc_small_fits<T>(m, n, wsum)) {
     task_trunc_small(c, t, smem, wsum);

@@ -48,7 +48,7 @@ struct ExecArgs {
   int64_t trunc_rows;           // rows of the truncation stacks in the scratch
   int32_t* status;              // [0] status code, [1] failing slot, [2] rank-cap hits, [3] abort,
                                 // [4] largest rank a truncation asked for (kRankMax + 1: more),
-                                // [5] dense-route truncations handed to the stack route
+                                // [5] dense- or sampled-route truncations handed to the stack route
   double* flops;                // accumulated algorithmic flops (may be null)
   unsigned long long wait_limit_ns;
   double jacobi_tol;            // truncation: Jacobi orthogonality tolerance
@@ -113,13 +113,14 @@ cudaError_t invert_blocks(const InvUnit* units, int32_t n_units, const InvLeaf* 
 
 constexpr int kExecThreads = 256;
 constexpr int kTruncStack = 96;  // columns of a truncation stack; wider pieces are stacked in parts
-// per-CTA scratch: two stacks (kTruncStack wide) and two outputs (kRankMax wide)
+// per-CTA scratch: two stacks (kTruncStack wide) and two outputs (kRankMax
+// wide), or the sampled route's four bases and its projections (1024 x 96)
 #ifdef __CUDACC__
 #define HLU_HD __host__ __device__
 #else
 #define HLU_HD
 #endif
-HLU_HD inline int64_t trunc_scratch_elems(int64_t rows) { return rows * (2 * kTruncStack + 2 * kRankMax); }
+HLU_HD inline int64_t trunc_scratch_elems(int64_t rows) { return rows * (2 * kTruncStack + 2 * kRankMax) + 1024 * 96; }
 inline int64_t trunc_scratch_bytes(int64_t rows, int elem_size) {
   int64_t b = trunc_scratch_elems(rows) * elem_size;
   return (b + 255) & ~int64_t(255);

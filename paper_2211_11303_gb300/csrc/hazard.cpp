@@ -263,7 +263,17 @@ class HazardCheck {
       case TK_PROJ: count(t.a); count(t.b); view(t.a); view(t.b); if (t.flags & TF_ADD) view(t.c); break;
       case TK_ROWMV: count(t.b); terms(t); if (!(t.flags & TF_OVERWRITE)) view(t.c); break;
       case TK_TRUNC: pieces(t); break;
-      case TK_DADD: count(t.c); count(t.a); view(t.a); view(t.b); if (!(t.flags & TF_OVERWRITE)) view(t.c); break;
+      case TK_DADD:
+        count(t.c);
+        if (t.flags & TF_PIECES) {
+          pieces(t);
+        } else {
+          count(t.a);
+          view(t.a);
+          view(t.b);
+        }
+        if (!(t.flags & TF_OVERWRITE)) view(t.c);
+        break;
       case TK_FENCE: break;
       default: throw std::logic_error("task type");
     }

@@ -45,7 +45,9 @@ enum TaskType : int32_t {
   TK_PROJ = 4,    // c (r x k) <- a^T b  (a: m x r, b: m x k)
   TK_ROWMV = 5,   // c (n x k) <- [c] + sign * sum_terms A_t B_t
   TK_TRUNC = 6,   // (a, b) <- truncate(sum_pieces sign X Y^T) to eps, rank -> out_slot
-  TK_DADD = 7,    // c (m x n) <- [c] + sign * a b^T  (a: m x k, b: n x k)
+  TK_DADD = 7,    // c (m x n) <- [c] + sign * a b^T  (a: m x k, b: n x k), or (TF_PIECES)
+                  // c <- [c] + sum_pieces sign X Y^T, c the window at (a.rows, a.cols) of the
+                  // target that the pieces' offsets refer to
   // 8: no longer used (its row of the executor's profile stays, empty)
   TK_NUM = 9,
   TK_FENCE = 9    // no work: orders re-use of temporary memory after its readers
@@ -53,13 +55,15 @@ enum TaskType : int32_t {
 // TF_ALPHA (DADD) and PF_ALPHA (a TRUNC piece): the sign is multiplied by the
 // launch's scalar alpha (the Schulz start X_0 = alpha A).  TF_ADD (PROJ of the
 // triangular solve): c += a^T b instead of c = a^T b.
-enum : int32_t { TF_OVERWRITE = 1, TF_ALPHA = 4, TF_ADD = 8 };
-enum : int32_t { PF_ALPHA = 1 };
+// PF_DENSE: the piece is the dense m x n matrix X over the whole target (Y is the
+// identity, for the routes that take factors).
+enum : int32_t { TF_OVERWRITE = 1, TF_ALPHA = 4, TF_ADD = 8, TF_PIECES = 16 };
+enum : int32_t { PF_ALPHA = 1, PF_DENSE = 2 };
 
 struct Task {
   int32_t type;
   int32_t flags;
-  int32_t list_begin, list_count;  // ROWMV terms or TRUNC pieces
+  int32_t list_begin, list_count;  // ROWMV terms, TRUNC or DADD pieces
   View a, b, c;
   int64_t piv_off;   // pivot vector offset (int32 elements) for leaf tasks
   int32_t out_slot;  // rank slot written by the task (-1: none)
@@ -75,7 +79,7 @@ struct Term {
   int32_t roff;
   int32_t pad;
 };
-// TRUNC piece: sign * X Y^T placed at rows [xoff, xoff + X.rows) of the target
+// TRUNC or DADD piece: sign * X Y^T placed at rows [xoff, xoff + X.rows) of the target
 // and columns [yoff, yoff + Y.rows); pad holds PF_ flags.
 struct Piece {
   View X, Y;

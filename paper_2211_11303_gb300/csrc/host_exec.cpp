@@ -138,6 +138,23 @@ void h_rowmv(HostCtx<T>& c, const Task& t) {
 
 template <class T>
 void h_dadd(HostCtx<T>& c, const Task& t) {
+  if (t.flags & TF_PIECES) {
+    const int wi = t.a.rows, wj = t.a.cols;
+    if (t.flags & TF_OVERWRITE)
+      for (int j = 0; j < t.c.cols; ++j)
+        for (int i = 0; i < t.c.rows; ++i) at(c, t.c, i, j) = T(0);
+    for (int q = 0; q < t.list_count; ++q) {
+      const Piece& P = c.pieces[t.list_begin + q];
+      const int w = ncols(c, P.X);
+      for (int j = std::max(P.yoff, wj); j < std::min(P.yoff + P.Y.rows, wj + t.c.cols); ++j)
+        for (int i = std::max(P.xoff, wi); i < std::min(P.xoff + P.X.rows, wi + t.c.rows); ++i) {
+          T s = 0;
+          for (int l = 0; l < w; ++l) s += at(c, P.X, i - P.xoff, l) * at(c, P.Y, j - P.yoff, l);
+          at(c, t.c, i - wi, j - wj) += T(P.sign) * s;
+        }
+    }
+    return;
+  }
   int m = t.c.rows, n = ncols(c, t.c), k = ncols(c, t.a);
   T sg = (t.flags & TF_ALPHA) ? T(t.sign) * T(c.alpha) : T(t.sign);
   for (int j = 0; j < n; ++j)
