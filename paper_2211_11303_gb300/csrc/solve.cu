@@ -3,7 +3,7 @@
 // application x = U^-1 (L^-1 P b) with up to 16 right-hand sides at a time.
 //
 // Every task is a narrow product: PROJ t (+)= Y^T z over a range of rows, or
-// ROWMV, one unit of at most 64 rows receiving sum_t A_t B_t (dense tiles,
+// ROWMV, one unit of at most 64 rows (mostly at most 32) receiving sum_t A_t B_t (dense tiles,
 // low-rank X factors, or a row panel of an inverted diagonal block).  The
 // work is one pass over the factor; what bounds it is the chain through the
 // solve blocks, three dependent tasks (panel, projection, update) per block
@@ -12,10 +12,10 @@
 // - Tasks are numbered in the order in which a simulated list schedule starts
 //   them and handed out by one counter per problem, so a CTA holds its task
 //   long before the task is ready.  It loads the task's records, builds the
-//   table of its columns and loads the first 32 columns of each warp into
-//   registers, and only then waits for the predecessors' counter.
-// - A finished task decrements its successors' counters with release
-//   reductions (no fence, no queue, no reply to wait for).
+//   table of its columns, loads the first 32 columns of each warp into registers
+//   and asks L2 for the others, and only then waits for the predecessors' counter.
+// - A finished task decrements its successors' counters with reductions after
+//   one fence (no queue, no reply to wait for).
 // - Lanes own rows (or, for PROJ, the summed index) and carry 4 or 8
 //   right-hand sides in registers; the eight warps split the columns and meet
 //   in shared memory.  The sums' order depends on neither the number of
@@ -27,7 +27,7 @@
 // resident together.  Every wait is bounded by the launch's limit
 // (%globaltimer); one that runs out records HLU_ERR_TIMEOUT and all CTAs stop.
 //
-// One apply of 8 columns at n = 24 (N = 91,656): 8.8 ms, against 54.8 ms for
+// One apply of 8 columns at n = 24 (N = 91,656): 7.8 ms, against 54.8 ms for
 // the tile-by-tile chain through the factorisation's executor.
 #include <cuda_runtime.h>
 
@@ -56,8 +56,9 @@ __device__ __forceinline__ int32_t ld_acquire_s32(const int32_t* p) {
   asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void red_release_dec(int32_t* p) {
-  asm volatile("red.release.gpu.global.add.s32 [%0], -1;" ::"l"(p) : "memory");
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void red_dec(int32_t* p) {
+  asm volatile("red.relaxed.gpu.global.add.s32 [%0], -1;" ::"l"(p) : "memory");
 }
 
 template <class T, int KC>
@@ -123,7 +124,7 @@ __device__ __forceinline__ T warp_halve(T (&v)[V], int lane) {
 // take the KC values of a row, so the shared stores are conflict-free
 template <class T, int KC, class At>
 __device__ __forceinline__ void stage_rows(T* b, int n, int kc, const At& at) {
-  constexpr int U = 8;
+  constexpr int U = KC * kCols / kThreads < 12 ? KC * kCols / kThreads : 12;
   for (int e0 = threadIdx.x; e0 < n * KC; e0 += U * kThreads) {
     T v[U];
 #pragma unroll
@@ -212,11 +213,15 @@ __device__ __forceinline__ void fill_columns(SolveSmem<T, KC>& s, int q0, int ba
   __syncthreads();
 }
 
-// One ROWMV task: unit rows r (lanes r and r + 32) of c, KC columns at a time.
-template <class T, int KC>
-__device__ bool run_rowmv(SolveSmem<T, KC>& s, const SolveProb& P, const SolveArgs& a) {
+// One ROWMV task: unit rows r (lane r, and r + 32 when NR is 2) of c, KC columns
+// at a time.  NR is a template parameter because a test of it between the
+// loads kept them from being in flight together (n = 24: 12.3 instead of
+// 8.4 ms an apply).
+template <class T, int KC, int NR>
+__device__ __forceinline__ bool run_rowmv(SolveSmem<T, KC>& s, const SolveProb& P, const SolveArgs& a) {
   constexpr int U = sizeof(T) == 4 ? 16 : 8;  // columns of a warp in one register buffer
   constexpr int kOut = 64 * KC / kThreads;    // outputs of a thread: row e % 64, column e / 64
+  constexpr int kLines = 64 * (int)sizeof(T) / 128;  // cache lines of a column
   T* arena = reinterpret_cast<T*>(P.arena);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rows = s.t.c.rows, k = P.nrhs;
@@ -226,9 +231,9 @@ __device__ bool run_rowmv(SolveSmem<T, KC>& s, const SolveProb& P, const SolveAr
   for (int j0 = 0; j0 < k; j0 += KC) {
     const int kc = min(KC, k - j0);
     T* out = arena + s.t.c.off + (int64_t)j0 * s.t.c.cs;
-    T acc[2][KC], old[kOut];
+    T acc[NR][KC], old[kOut];
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < NR; ++i)
 #pragma unroll
       for (int j = 0; j < KC; ++j) acc[i][j] = T(0);
     bool have_old = false;
@@ -245,38 +250,46 @@ __device__ bool run_rowmv(SolveSmem<T, KC>& s, const SolveProb& P, const SolveAr
       for (int base = 0; base < total; base += kCols) {
         const int n = min(kCols, total - base);
         fill_columns(s, q0, base);
-        // buffer g holds columns warp + 8 (g U + u) of the chunk
-        T x[2][U], y[2][U];
-        auto load = [&](T(&v)[2][U], int g) {
+        // buffer g holds columns warp + 8 (g U + u) of the chunk; lanes and
+        // columns outside repeat an element inside and count it as zero, so
+        // that no branch comes between the loads
+        T x[NR][U], y[NR][U];
+        auto load = [&](T(&v)[NR][U], int g) {
 #pragma unroll
           for (int u = 0; u < U; ++u) {
-            const int c = warp + kWarps * (g * U + u);
-            v[0][u] = v[1][u] = T(0);
-            if (c < n) {
-              const int r = s.col_r[c], lo = r & 255, hi = r >> 8;
-              const T* p = arena + s.col_a[c];
-              if (lane >= lo && lane < hi) v[0][u] = __ldg(p + lane);
-              if (lane + 32 >= lo && lane + 32 < hi) v[1][u] = __ldg(p + lane + 32);
+            const int c = warp + kWarps * (g * U + u), cc = min(c, n - 1);
+            const int r = s.col_r[cc], lo = r & 255, hi = r >> 8;
+            const T* p = arena + s.col_a[cc];
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+              const int row = lane + 32 * i;
+              const T q = __ldg(p + min(max(row, lo), hi - 1));
+              v[i][u] = c < n && row >= lo && row < hi ? q : T(0);
             }
           }
         };
-        auto fma = [&](const T(&v)[2][U], int g) {
+        auto fma = [&](const T(&v)[NR][U], int g) {
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             const int c = warp + kWarps * (g * U + u);
-            if (c < n) {
-              T w[KC];
-              row_of<KC>(s.b + c * KC, w);
+            if (sizeof(T) == 8 && c >= n) continue;  // FP64 is bound by its FMAs
+            T w[KC];
+            row_of<KC>(s.b + min(c, n - 1) * KC, w);
 #pragma unroll
-              for (int j = 0; j < KC; ++j) {
-                acc[0][j] += v[0][u] * w[j];
-                acc[1][j] += v[1][u] * w[j];
-              }
-            }
+            for (int i = 0; i < NR; ++i)
+#pragma unroll
+              for (int j = 0; j < KC; ++j) acc[i][j] += v[i][u] * w[j];
           }
         };
+        const int groups = (n + kWarps * U - 1) / (kWarps * U);
         load(x, 0);
-        load(y, 1);
+        if (groups > 1) load(y, 1);
+        // the columns behind the registers come from L2 then, not from memory
+        for (int e = threadIdx.x; e < (n - 2 * kWarps * U) * kLines; e += kThreads) {
+          const int c = 2 * kWarps * U + e / kLines, r = s.col_r[c], lo = r & 255, hi = r >> 8;
+          const int row = lo + (e % kLines) * (128 / (int)sizeof(T));
+          if (row < hi) prefetch_l2(arena + s.col_a[c] + row);
+        }
         if (!waited) {
           if (!wait_ready(s, P, a)) return false;
           waited = true;
@@ -284,7 +297,6 @@ __device__ bool run_rowmv(SolveSmem<T, KC>& s, const SolveProb& P, const SolveAr
         if (!have_old) load_old();
         stage_rows<T, KC>(s.b, n, kc, [&](int c, int j) { return arena + s.col_b[c] + (int64_t)(j0 + j) * s.col_ld[c]; });
         __syncthreads();
-        const int groups = (n + kWarps * U - 1) / (kWarps * U);
         for (int g = 0; g < groups; g += 2) {
           fma(x, g);
           if (g + 2 < groups) load(x, g + 2);
@@ -303,16 +315,17 @@ __device__ bool run_rowmv(SolveSmem<T, KC>& s, const SolveProb& P, const SolveAr
     // the warps' partial sums: [warp][j][row]
 #pragma unroll
     for (int j = 0; j < KC; ++j) {
-      s.b[(warp * KC + j) * 64 + lane] = acc[0][j];
-      s.b[(warp * KC + j) * 64 + lane + 32] = acc[1][j];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) s.b[(warp * KC + j) * 64 + lane + 32 * i] = acc[i][j];
     }
     __syncthreads();
 #pragma unroll
     for (int o = 0; o < kOut; ++o) {
       const int e = threadIdx.x + o * kThreads, r = e & 63, j = e >> 6;
       T sum = T(0);
+      if (r < rows)
 #pragma unroll
-      for (int w = 0; w < kWarps; ++w) sum += s.b[w * KC * 64 + e];
+        for (int w = 0; w < kWarps; ++w) sum += s.b[w * KC * 64 + e];
       if (r < rows && j < kc) __stcg(out + r + (int64_t)j * s.t.c.cs, old[o] + sign * sum);
     }
     __syncthreads();
@@ -351,6 +364,12 @@ __device__ bool run_proj(SolveSmem<T, KC>& s, const SolveProb& P, const SolveArg
   };
   if (busy && pair0 < npairs) load(x, pair0, 0, sub);
   bool preloaded = true;
+  {
+    const int lines = (m * (int)sizeof(T) + 127) / 128, per = 128 / (int)sizeof(T);
+    for (int e = threadIdx.x; e < r * lines; e += kThreads)
+      if (e / lines >= 2 * kWarps || (e % lines) * per >= 32 * U * split)
+        prefetch_l2(A + (int64_t)(e / lines) * lda + (e % lines) * per);
+  }
   if (!wait_ready(s, P, a)) return false;
   for (int j0 = 0; j0 < k; j0 += KC) {
     const int kc = min(KC, k - j0);
@@ -447,22 +466,25 @@ __global__ void __launch_bounds__(kThreads, 2) solve_kernel(const __grid_constan
       reinterpret_cast<int32_t*>(&s.t)[threadIdx.x] = __ldg(reinterpret_cast<const int32_t*>(P.tasks + ti) + threadIdx.x);
     if (threadIdx.x >= 64 && threadIdx.x < 66) s.succ[threadIdx.x - 64] = __ldg(P.succ_ptr + ti + threadIdx.x - 64);
     __syncthreads();
-    // warp 0 also holds the first 32 successors
+    // every thread holds one of the first 256 successors
     const int64_t e0 = s.succ[0], e1 = s.succ[1];
     int32_t sx = -1;
-    if (threadIdx.x < 32 && e0 + threadIdx.x < e1) sx = __ldg(P.succ_idx + e0 + threadIdx.x);
+    if (e0 + threadIdx.x < e1) sx = __ldg(P.succ_idx + e0 + threadIdx.x);
     bool ok;
     if (s.t.type == TK_PROJ)
       ok = run_proj<T, KC>(s, P, a);
     else if (s.t.type == TK_ROWMV)
-      ok = run_rowmv<T, KC>(s, P, a);
+      ok = s.t.c.rows <= 32 ? run_rowmv<T, KC, 1>(s, P, a) : run_rowmv<T, KC, 2>(s, P, a);
     else
       ok = wait_ready(s, P, a);
     if (!ok) break;
     __syncthreads();  // the task's stores come before the releases
-    if (threadIdx.x < 32) {
-      if (sx >= 0) red_release_dec(P.indeg + sx);
-      for (int64_t e = e0 + 32 + threadIdx.x; e < e1; e += 32) red_release_dec(P.indeg + __ldg(P.succ_idx + e));
+    // one fence a thread, then plain reductions (a release per reduction waited
+    // for the stores again every 32 successors)
+    if (sx >= 0) {
+      __threadfence();
+      red_dec(P.indeg + sx);
+      for (int64_t e = e0 + kThreads + threadIdx.x; e < e1; e += kThreads) red_dec(P.indeg + __ldg(P.succ_idx + e));
     }
     if (a.trace && threadIdx.x == 0) {
       unsigned long long* tr = a.trace + 4 * ti;
