@@ -2402,11 +2402,15 @@ __device__ bool task_trunc_sampled(Ctx<T>& c, const Task& t, char* smem, int W) 
   expand(xat, sm.xlo, sm.xhi, m, k, S);
   lap(0);
   const T f2 = T(0.01 * c.eps * c.eps);
+  // the steps also end at the rounding of the samples, five units (FP32 at
+  // eps 1e-6: 0.3 eps); beyond it the pivots are noise
+  const T noise = sizeof(T) == 4 ? T(9e-14) : T(3e-31);
+  const T floor2 = max(f2, noise);
   T tail = 0, first = 0;
   const int kend = min(min(k - 6, 64), min(m, n));
   const int rp = mgs_columns(
       S, m, k, kend, S1, sm, (T*)nullptr,
-      [&](int j, T tl, T fst) { return tl * T(k) <= f2 * fst * T(k - j); }, &tail, &first);
+      [&](int j, T tl, T fst) { return tl * T(k) <= floor2 * fst * T(k - j); }, &tail, &first);
   if (rp == kend) {
     // (sm.inv holds 1 / pivot norm)
     const T miss = tail * T(k) / (f2 * first * T(k - rp));  // (missed / 0.1 eps s_1)^2
@@ -2501,8 +2505,8 @@ __device__ void task_trunc(Ctx<T>& c, const Task& t, char* smem) {
     return;
   }
   if (m <= kDenseMax && n <= kDenseMax && task_trunc_dense(c, t, smem)) return;
-  // below kRsEps the floor is under the rounding of the samples
-  constexpr double kRsEps = sizeof(T) == 4 ? 4e-6 : 1e-13;
+  // below kRsEps the rounding of the samples is above eps
+  constexpr double kRsEps = sizeof(T) == 4 ? 5e-7 : 1e-13;
   if (wsum > kRsMin && wsum <= kRsCols && t.list_count <= kRsPieces && min(m, n) >= 64 && c.eps >= kRsEps &&
       task_trunc_sampled(c, t, smem, wsum))
     return;
