@@ -1187,6 +1187,8 @@ static int factor_prepare(hlu_handle* h, int32_t precision, cudaStream_t s) {
     CKR(dev_malloc(&h->d_arena, (size_t)es * h->L.total), "arena");
     CKR(dev_malloc(&h->d_ranks, sizeof(int32_t) * std::max(h->L.n_slots, 1)), "ranks");
     CKR(dev_malloc(&h->d_piv, sizeof(int32_t) * std::max<int64_t>(h->L.piv_total, 1)), "piv");
+    // row numbers of their tiles from the first launch on, whatever part of it runs
+    CKR(cudaMemsetAsync(h->d_piv, 0, sizeof(int32_t) * std::max<int64_t>(h->L.piv_total, 1), s), "piv");
     CKR(dev_malloc(&h->d_scratch, (size_t)es * h->scratch_stride * h->grid), "scratch");
     CKR(dev_malloc(&h->d_status, sizeof(int32_t) * 8), "status");
     CKR(dev_malloc(&h->d_flops, sizeof(double)), "flops");
@@ -1216,15 +1218,18 @@ static int factor_prepare(hlu_handle* h, int32_t precision, cudaStream_t s) {
   return HLU_OK;
 }
 
-// after a factorisation was launched: the solve blocks' inverses
-static int factor_inverses(hlu_handle* h, cudaStream_t s) {
+// after a factorisation was launched: the solve blocks' inverses (status_of:
+// the handle whose status words the launch uses)
+static int factor_inverses(hlu_handle* h, const hlu_handle* status_of, cudaStream_t s) {
   const SchedBundle& b = *h->sb;
   const int32_t nu = (int32_t)b.L.inv_units.size(), nl = (int32_t)b.L.inv_leaves.size();
   if (h->precision == HLU_FP64)
-    CKR(invert_blocks<double>(b.d_inv_units, nu, b.d_inv_leaves, nl, (double*)h->d_arena, h->d_ranks, h->d_piv, s),
+    CKR(invert_blocks<double>(b.d_inv_units, nu, b.d_inv_leaves, nl, (double*)h->d_arena, h->d_ranks, h->d_piv,
+                              status_of->d_status, s),
         "solve blocks");
   else
-    CKR(invert_blocks<float>(b.d_inv_units, nu, b.d_inv_leaves, nl, (float*)h->d_arena, h->d_ranks, h->d_piv, s),
+    CKR(invert_blocks<float>(b.d_inv_units, nu, b.d_inv_leaves, nl, (float*)h->d_arena, h->d_ranks, h->d_piv,
+                             status_of->d_status, s),
         "solve blocks");
   return HLU_OK;
 }
@@ -1279,7 +1284,7 @@ static int factor_impl(hlu_handle* h, int32_t precision, void* stream, int64_t l
     CKR(cudaEventRecord(h->ev0, s), "event");
     rc = exec_run(h, h->dF, h->grid, s, true, limit);
     if (rc) return rc;
-    if (limit < 0 && (rc = factor_inverses(h, s))) return rc;
+    if (limit < 0 && (rc = factor_inverses(h, h, s))) return rc;
     CKR(cudaEventRecord(h->ev1, s), "event");
     CKR(cudaEventSynchronize(h->ev1), "sync");
     float ms = 0;
@@ -1304,7 +1309,7 @@ int hlu_factor_async(hlu_handle* h, int32_t precision, int32_t max_ctas, void* s
     const int grid = max_ctas > 0 ? std::min(h->grid, (int)max_ctas) : h->grid;
     rc = exec_run(h, h->dF, grid, s, true);
     if (rc) return rc;
-    if ((rc = factor_inverses(h, s))) return rc;
+    if ((rc = factor_inverses(h, h, s))) return rc;
     CKR(cudaEventRecord(h->ev1, s), "event");
     h->factor_pending = true;
     h->factor_stream = s;
@@ -1695,7 +1700,7 @@ int hlu_factor_batch(hlu_handle** hs, int32_t count, int32_t precision, void* st
     int rc = exec_run_batch(hs, count, s, &g_batch_q, &g_batch_q_len);
     if (rc) return rc;
     for (int32_t i = 0; i < count; ++i)
-      if ((rc = factor_inverses(hs[i], s))) return rc;
+      if ((rc = factor_inverses(hs[i], hs[0], s))) return rc;
     CKR(cudaEventRecord(hs[0]->ev1, s), "event");
     CKR(cudaEventSynchronize(hs[0]->ev1), "sync");
     float ms = 0;

@@ -2810,9 +2810,15 @@ cudaError_t tc_tile_product(const float* A, const float* B, float* D, int K, int
 
 #if !HLU_EXEC_TC
 // ---------------------------------------------------------------- solve blocks
+// Both kernels follow the executor's launch on its stream, before the host has
+// read that launch's status.  A launch whose wait ran out (status[3]) leaves
+// factors and pivots unwritten: nothing is inverted then.
+
 // Dense copies of the solve blocks' diagonal blocks: one CTA per leaf block.
 template <class T>
-__global__ void __launch_bounds__(NT) k_inv_copy(const InvLeaf* leaves, T* arena, const int32_t* ranks) {
+__global__ void __launch_bounds__(NT)
+    k_inv_copy(const InvLeaf* leaves, T* arena, const int32_t* ranks, const int32_t* status) {
+  if (status[3]) return;
   const InvLeaf f = leaves[blockIdx.x];
   const int r = f.slot < 0 ? 0 : ranks[f.slot];
   for (int64_t e = threadIdx.x; e < (int64_t)f.m * f.n; e += NT) {
@@ -2858,7 +2864,9 @@ struct InvCursor {
 // columns per warp (one per right-hand side of the substitution), the pivot
 // tile and the right-hand sides in shared memory.
 template <class T>
-__global__ void __launch_bounds__(NT) k_inv_units(const InvUnit* units, T* arena, const int32_t* piv) {
+__global__ void __launch_bounds__(NT)
+    k_inv_units(const InvUnit* units, T* arena, const int32_t* piv, const int32_t* status) {
+  if (status[3]) return;
   extern __shared__ __align__(16) char smem[];
   T* As = reinterpret_cast<T*>(smem);
   T* Bs = As + kStage;
@@ -2930,20 +2938,20 @@ __global__ void __launch_bounds__(NT) k_inv_units(const InvUnit* units, T* arena
 
 template <class T>
 cudaError_t invert_blocks(const InvUnit* units, int32_t n_units, const InvLeaf* leaves, int32_t n_leaves, T* arena,
-                          const int32_t* ranks, const int32_t* piv, cudaStream_t s) {
+                          const int32_t* ranks, const int32_t* piv, const int32_t* status, cudaStream_t s) {
   const size_t sm = sizeof(T) * (2 * kStage + 64 * 64 + 65 * 64);
   cudaError_t e = cudaFuncSetAttribute(k_inv_units<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess || n_units == 0) return e;
   note_launch();
-  k_inv_copy<T><<<n_leaves, NT, 0, s>>>(leaves, arena, ranks);
+  k_inv_copy<T><<<n_leaves, NT, 0, s>>>(leaves, arena, ranks, status);
   note_launch();
-  k_inv_units<T><<<dim3(n_units, 2), NT, sm, s>>>(units, arena, piv);
+  k_inv_units<T><<<dim3(n_units, 2), NT, sm, s>>>(units, arena, piv, status);
   return cudaGetLastError();
 }
 template cudaError_t invert_blocks<float>(const InvUnit*, int32_t, const InvLeaf*, int32_t, float*, const int32_t*,
-                                          const int32_t*, cudaStream_t);
+                                          const int32_t*, const int32_t*, cudaStream_t);
 template cudaError_t invert_blocks<double>(const InvUnit*, int32_t, const InvLeaf*, int32_t, double*, const int32_t*,
-                                           const int32_t*, cudaStream_t);
+                                           const int32_t*, const int32_t*, cudaStream_t);
 #endif
 
 size_t exec_smem_bytes(int elem_size) {

@@ -106,10 +106,11 @@ cudaError_t solve_launch(SolveArgs& a, cudaStream_t s);
 
 // Inverts the triangular factors of every solve block of a factored arena
 // (exec.cu): dense copies of the diagonal blocks, then one CTA per unit and
-// triangle.
+// triangle.  status: the factorisation's status words; nothing runs when its
+// abort flag (status[3]) is set.
 template <class T>
 cudaError_t invert_blocks(const InvUnit* units, int32_t n_units, const InvLeaf* leaves, int32_t n_leaves, T* arena,
-                          const int32_t* ranks, const int32_t* piv, cudaStream_t s);
+                          const int32_t* ranks, const int32_t* piv, const int32_t* status, cudaStream_t s);
 
 constexpr int kExecThreads = 256;
 constexpr int kTruncStack = 96;  // columns of a truncation stack; wider pieces are stacked in parts

@@ -188,3 +188,53 @@ def test_library_memory_comes_from_torch(hlu):
     finally:
         hlu.hlu_destroy(h)
     assert hlu.hlu_device_bytes_in_use() == before_l
+
+
+@pytest.mark.parametrize("call", ["factor", "async", "batch"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_factorisation_whose_wait_runs_out(hlu, call, prec):
+    """A factorisation that stops half way (CTAs wait far longer than 20 us for
+    a ready task) inverts no solve block from pivots it never wrote, reports
+    the timeout, and the same handle factors and solves afterwards as one that
+    never failed."""
+    P = hlu.HLU_FP64 if prec == "fp64" else hlu.HLU_FP32
+    # recycled blocks of the caching allocator: no pivot is a row number by luck
+    for nbytes in [1 << k for k in range(9, 22)]:
+        torch.full((nbytes,), 0x7F, dtype=torch.uint8, device="cuda")
+    hs = [hlu.hlu_build(n, 3.0, 16, 2.0, 1e-6) for n in ((6, 5) if call == "batch" else (6,))]
+
+    def factor():
+        if call == "batch":
+            hlu.hlu_factor_batch(hs, P)
+        elif call == "async":
+            hlu.hlu_factor_async(hs[0], P)
+            hlu.hlu_factor_wait(hs[0], block=True)
+        else:
+            hlu.hlu_factor(hs[0], P)
+
+    try:
+        hlu.hlu_set_wait_limit_ms(0.02)
+        try:
+            with pytest.raises(hlu.HluError) as ei:
+                factor()
+        finally:
+            hlu.hlu_set_wait_limit_ms(20000)
+        assert ei.value.status == "HLU_ERR_TIMEOUT"
+        torch.cuda.synchronize()
+        factor()
+        for h in hs:
+            N = hlu.hlu_n(h)
+            b = torch.from_numpy(synth.normal(3, N)).cuda()
+            x = torch.empty_like(b)
+            hlu.hlu_solve(h, b, x)
+            fresh = hlu.hlu_build(6 if h == hs[0] else 5, 3.0, 16, 2.0, 1e-6)
+            try:
+                y = torch.empty_like(b)
+                hlu.hlu_factor(fresh, P)
+                hlu.hlu_solve(fresh, b, y)
+                assert torch.equal(x, y)
+            finally:
+                hlu.hlu_destroy(fresh)
+    finally:
+        for h in hs:
+            hlu.hlu_destroy(h)
