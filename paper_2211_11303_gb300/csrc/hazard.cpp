@@ -305,9 +305,9 @@ class HazardCheck {
 
 }  // namespace
 
-extern "C" int hlu_debug_check_hazards(int32_t nc, const int32_t* clusters, int32_t nb, const int32_t* blocks,
-                                       int32_t rank_cap, int32_t tile, int32_t nrhs_max, int32_t which,
-                                       int64_t drop_edge, int64_t* report) {
+static int check_hazards(int32_t nc, const int32_t* clusters, int32_t nb, const int32_t* blocks, int32_t rank_cap,
+                         int32_t tile, int32_t nrhs_max, int32_t which, int64_t drop_edge, int64_t ring,
+                         int64_t* report, SchedStats& st) {
   try {
     if (!clusters || !blocks || !report || nc < 1 || nb < 1 || nrhs_max < 1 || nrhs_max > 16 || which < 0 ||
         which > 4 || rank_cap < 0 || rank_cap > kRankMax)
@@ -318,15 +318,14 @@ extern "C" int hlu_debug_check_hazards(int32_t nc, const int32_t* clusters, int3
     trees_from_export(nc, clusters, nb, blocks, C, B);
     const int32_t cap = rank_cap > 0 ? rank_cap : kRankMax;
     ArenaLayout L;
-    SchedStats st;
     Schedule F, S, S0, S1, S2;
     Schedule* pick = nullptr;
     if (which <= 1) {
-      build_schedules(C, B, cap, nrhs_max, tile, L, F, S, st, nullptr);
+      build_schedules(C, B, cap, nrhs_max, tile, L, F, S, st, nullptr, ring);
       pick = which == 0 ? &F : &S;
     } else {
       std::vector<Block> FB = factor_tree(C, B, tile), Bx;
-      build_inverse_schedules(C, FB, cap, nrhs_max, tile, L, Bx, S0, S1, S2, st);
+      build_inverse_schedules(C, FB, cap, nrhs_max, tile, L, Bx, S0, S1, S2, st, ring);
       pick = which == 2 ? &S0 : which == 3 ? &S1 : &S2;
     }
     if (drop_edge >= (int64_t)pick->pred_idx.size()) return 1;
@@ -348,4 +347,22 @@ extern "C" int hlu_debug_check_hazards(int32_t nc, const int32_t* clusters, int3
   } catch (const std::exception&) {
     return 6;
   }
+}
+
+extern "C" int hlu_debug_check_hazards(int32_t nc, const int32_t* clusters, int32_t nb, const int32_t* blocks,
+                                       int32_t rank_cap, int32_t tile, int32_t nrhs_max, int32_t which,
+                                       int64_t drop_edge, int64_t* report) {
+  SchedStats st;
+  return check_hazards(nc, clusters, nb, blocks, rank_cap, tile, nrhs_max, which, drop_edge, 0, report, st);
+}
+
+extern "C" int hlu_debug_check_hazards_ring(int32_t nc, const int32_t* clusters, int32_t nb, const int32_t* blocks,
+                                            int32_t rank_cap, int32_t tile, int32_t nrhs_max, int32_t which,
+                                            int64_t ring, int64_t* report) {
+  if (ring < 0 || !report) return 1;
+  SchedStats st;
+  report[11] = 0;
+  const int rc = check_hazards(nc, clusters, nb, blocks, rank_cap, tile, nrhs_max, which, -1, ring, report, st);
+  if (rc == 0 || rc == 9) report[11] = st.ring_wraps;
+  return rc;
 }

@@ -156,10 +156,12 @@ struct SchedStats {
 // `tile`: every block-tree node whose row and column clusters both hold at most
 // `tile` DOFs is factored as one dense tile (tile <= leaf keeps the block tree
 // as it is).  factor_blocks (optional) receives the factor tree the schedules
-// and the arena layout refer to.
+// and the arena layout refer to.  ring_elems: size of the region for
+// temporaries (0: by the factor's size); throws when it cannot hold them.
 void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& B, int32_t rank_cap,
                      int32_t nrhs_max, int32_t tile, ArenaLayout& L,
-                     Schedule& factor, Schedule& solve, SchedStats& st, std::vector<Block>* factor_blocks);
+                     Schedule& factor, Schedule& solve, SchedStats& st, std::vector<Block>* factor_blocks,
+                     int64_t ring_elems = 0);
 std::vector<Block> factor_tree(const std::vector<Cluster>& C, const std::vector<Block>& B, int32_t tile);
 
 // The Schulz iteration for the inverse of A_H (Sec. 3, Sec. 4) over four
@@ -171,6 +173,7 @@ std::vector<Block> factor_tree(const std::vector<Cluster>& C, const std::vector<
 // out_off).
 void build_inverse_schedules(const std::vector<Cluster>& C, const std::vector<Block>& FB, int32_t rank_cap,
                              int32_t nrhs_max, int32_t tile, ArenaLayout& L, std::vector<Block>& Bx,
-                             Schedule& start, Schedule& iter, Schedule& apply, SchedStats& st);
+                             Schedule& start, Schedule& iter, Schedule& apply, SchedStats& st,
+                             int64_t ring_elems = 0);
 
 }  // namespace hlu

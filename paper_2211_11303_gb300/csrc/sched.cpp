@@ -188,10 +188,6 @@ class Sched {
   static constexpr int64_t kBuckets = 64;
   int64_t ring_pos() const { return pass_ * ring_size_ + cursor_; }
   static int64_t position(const LR& p) { return std::min(p.X.at, p.Y.at); }
-  int64_t room(const LR& p) const {  // elements that can be allocated before p's memory is reused
-    const int64_t at = position(p);
-    return at == kNotTemp ? kNotTemp : at + ring_size_ - ring_pos();
-  }
   void add_old_pieces(int64_t n) {
     const int64_t bucket = (ring_size_ + kBuckets - 1) / kBuckets;
     const int64_t until = (ring_pos() + n - ring_size_ + ring_size_ / 4) / bucket;
@@ -254,6 +250,8 @@ class Sched {
       pending_fence_.clear();
     }
     for (int64_t ch = last_alloc_lo_; ch <= last_alloc_hi_; ++ch) chunk_occ_[ch].push_back(b);
+    buf_chunk_[b] = (int32_t)last_alloc_lo_;
+    buf_pass_[b] = pass_;
   }
   int32_t new_slot() { return L_.n_slots++; }
   int64_t temp_elems_ = 0;
@@ -264,6 +262,8 @@ class Sched {
     bufs_.push_back(b);
     acc_head_.push_back(-1);
     acc_last_.push_back(-1);
+    buf_chunk_.push_back(-1);
+    buf_pass_.push_back(0);
     fence_begin_.push_back(0);
     fence_end_.push_back(0);
     return (int32_t)bufs_.size() - 1;
@@ -383,8 +383,13 @@ class Sched {
     stamp_[p] = cur_;
     deps_.push_back(p);
   }
+  // A temporary may be used until its first chunk is entered in a later pass of
+  // the ring: the fence made then orders the chunk's next occupants after the
+  // accesses noted so far, and no later one.
   void note_access(int32_t b) {
     if (acc_last_[b] == cur_) return;
+    if (buf_chunk_[b] >= 0 && chunk_pass_[buf_chunk_[b]] != buf_pass_[b])
+      throw std::runtime_error("temporaries of one block's update exceed the ring");
     acc_last_[b] = cur_;
     grow4(acc_task_);
     grow4(acc_next_);
@@ -654,7 +659,6 @@ class Sched {
   // ---------------------------------------------------------------- truncation
   // one piece of a TRUNC or DADD task, with its reads
   void push_piece(const PieceMV& p, bool alpha) {
-    if (room(p.p) < 0) throw std::runtime_error("temporaries of one block's update exceed the ring");
     Piece q;
     std::memset(&q, 0, sizeof(q));
     q.X = p.p.X.v;
@@ -1262,6 +1266,7 @@ class Sched {
   std::vector<int32_t> fence_pool_;
   std::vector<int64_t> acc_head_;
   std::vector<int32_t> acc_last_;
+  std::vector<int32_t> buf_chunk_, buf_pass_;  // a temporary's first chunk (else -1) and its pass
   std::vector<int32_t> acc_task_;
   std::vector<int64_t> acc_next_;
   std::vector<int32_t> seg_buf_;
@@ -1468,7 +1473,7 @@ void order_for_tickets(Schedule& S) {
 void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bfull, int32_t rank_cap,
                      int32_t nrhs_max, int32_t tile, ArenaLayout& L,
                      Schedule& factor, Schedule& solve,
-                     SchedStats& st, std::vector<Block>* factor_blocks) {
+                     SchedStats& st, std::vector<Block>* factor_blocks, int64_t ring_elems) {
   std::vector<Block> Bt = factor_tree(C, Bfull, tile);
   const std::vector<Block>& B = Bt;
   if (factor_blocks) *factor_blocks = Bt;
@@ -1524,8 +1529,10 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bf
   // keeps the number of wraps (and fences) of the larger workloads at what a
   // 2^30 bound gave at capacity 32.
   const int64_t ring =
-      std::max(inv_scratch, std::min<int64_t>(std::max<int64_t>(8 * fe, int64_t(1) << 22), int64_t(1) << 31));
-  const int64_t ring_off = alloc(ring);
+      ring_elems > 0
+          ? ring_elems
+          : std::max(inv_scratch, std::min<int64_t>(std::max<int64_t>(8 * fe, int64_t(1) << 22), int64_t(1) << 31));
+  const int64_t ring_off = alloc(std::max(ring, inv_scratch));
   L.ring_off = ring_off;
   L.ring_size = ring;
   // the dense copies are scratch between the factorisation and the solves:
@@ -1561,7 +1568,8 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bf
 
 void build_inverse_schedules(const std::vector<Cluster>& C, const std::vector<Block>& FB, int32_t rank_cap,
                              int32_t nrhs_max, int32_t tile, ArenaLayout& L, std::vector<Block>& Bx,
-                             Schedule& start, Schedule& iter, Schedule& apply, SchedStats& st) {
+                             Schedule& start, Schedule& iter, Schedule& apply, SchedStats& st,
+                             int64_t ring_elems) {
   auto t0 = std::chrono::steady_clock::now();
   const int32_t nb = (int32_t)FB.size();
   Bx.assign((size_t)4 * nb, Block());
@@ -1611,7 +1619,8 @@ void build_inverse_schedules(const std::vector<Cluster>& C, const std::vector<Bl
   L.nrhs_slot = L.n_slots++;
   L.work_off = alloc((int64_t)C[0].size * nrhs_max);
   L.out_off = alloc((int64_t)C[0].size * nrhs_max);
-  const int64_t ring = std::min<int64_t>(std::max<int64_t>(8 * fe, int64_t(1) << 22), int64_t(1) << 31);
+  const int64_t ring =
+      ring_elems > 0 ? ring_elems : std::min<int64_t>(std::max<int64_t>(8 * fe, int64_t(1) << 22), int64_t(1) << 31);
   L.ring_off = alloc(ring);
   L.ring_size = ring;
   const int32_t segsz = std::max(leafmax, tile);
