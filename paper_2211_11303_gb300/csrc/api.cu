@@ -1005,7 +1005,8 @@ int hlu_build(const hlu_mesh* mesh, double kappa, int32_t leaf, double eta, doub
     uint64_t key = 1469598103934665603ULL;
     key = fnv1a(key, h->trees.clusters.data(), sizeof(int32_t) * h->trees.clusters.size());
     key = fnv1a(key, h->trees.blocks.data(), sizeof(int32_t) * h->trees.blocks.size());
-    int32_t params[4] = {rank_cap, h->tile, nrhs_max, (int32_t)N};
+    const bool accumulate = accumulate_updates(h->tile, eps);
+    int32_t params[5] = {rank_cap, h->tile, nrhs_max, (int32_t)N, accumulate ? 1 : 0};
     key = fnv1a(key, params, sizeof(params));
     bool cache_hit = false;
     {
@@ -1024,7 +1025,7 @@ int hlu_build(const hlu_mesh* mesh, double kappa, int32_t leaf, double eta, doub
       sb->key = key;
       Schedule F, S;
       build_schedules(h->C, h->B, rank_cap, nrhs_max, h->tile, sb->L, F, S, sb->st,
-                      &sb->FB);
+                      &sb->FB, accumulate);
       if ((e = sb->dF.load(F)) != cudaSuccess) return bail(e, "upload factor schedule");
       if ((e = sb->dS.load(S)) != cudaSuccess) return bail(e, "upload solve schedule");
       // A_H fill descriptors

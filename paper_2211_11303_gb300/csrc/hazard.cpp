@@ -306,8 +306,8 @@ class HazardCheck {
 }  // namespace
 
 static int check_hazards(int32_t nc, const int32_t* clusters, int32_t nb, const int32_t* blocks, int32_t rank_cap,
-                         int32_t tile, int32_t nrhs_max, int32_t which, int64_t drop_edge, int64_t ring,
-                         int64_t* report, SchedStats& st) {
+                         int32_t tile, int32_t nrhs_max, int32_t which, int64_t drop_edge, bool accumulate,
+                         int64_t ring, int64_t* report, SchedStats& st, int64_t* trunc_chain) {
   try {
     if (!clusters || !blocks || !report || nc < 1 || nb < 1 || nrhs_max < 1 || nrhs_max > 16 || which < 0 ||
         which > 4 || rank_cap < 0 || rank_cap > kRankMax)
@@ -321,7 +321,7 @@ static int check_hazards(int32_t nc, const int32_t* clusters, int32_t nb, const 
     Schedule F, S, S0, S1, S2;
     Schedule* pick = nullptr;
     if (which <= 1) {
-      build_schedules(C, B, cap, nrhs_max, tile, L, F, S, st, nullptr, ring);
+      build_schedules(C, B, cap, nrhs_max, tile, L, F, S, st, nullptr, accumulate, ring);
       pick = which == 0 ? &F : &S;
     } else {
       std::vector<Block> FB = factor_tree(C, B, tile), Bx;
@@ -339,6 +339,15 @@ static int check_hazards(int32_t nc, const int32_t* clusters, int32_t nb, const 
       --pick->n_edges;
     }
     const int64_t T = (int64_t)pick->tasks.size();
+    if (trunc_chain) {
+      std::vector<int64_t> chain(T, 0);  // truncations on the longest chain that ends with a task
+      for (int64_t t = 0; t < T; ++t) {
+        for (int64_t e = pick->pred_ptr[t]; e < pick->pred_ptr[t + 1]; ++e)
+          chain[t] = std::max(chain[t], chain[pick->pred_idx[e]]);
+        chain[t] += pick->tasks[t].type == TK_TRUNC;
+        *trunc_chain = std::max(*trunc_chain, chain[t]);
+      }
+    }
     if (T > 40000 || L.total > (int64_t)1 << 27) return 6;  // bitsets and element states stay in host memory
     HazardCheck hc(*pick, L.total, L.piv_total, L.n_slots, L.nrhs_slot);
     hc.run(report);
@@ -353,16 +362,22 @@ extern "C" int hlu_debug_check_hazards(int32_t nc, const int32_t* clusters, int3
                                        int32_t rank_cap, int32_t tile, int32_t nrhs_max, int32_t which,
                                        int64_t drop_edge, int64_t* report) {
   SchedStats st;
-  return check_hazards(nc, clusters, nb, blocks, rank_cap, tile, nrhs_max, which, drop_edge, 0, report, st);
+  return check_hazards(nc, clusters, nb, blocks, rank_cap, tile, nrhs_max, which, drop_edge, tile > 0, 0, report, st,
+                       nullptr);
 }
 
 extern "C" int hlu_debug_check_hazards_ring(int32_t nc, const int32_t* clusters, int32_t nb, const int32_t* blocks,
                                             int32_t rank_cap, int32_t tile, int32_t nrhs_max, int32_t which,
-                                            int64_t ring, int64_t* report) {
-  if (ring < 0 || !report) return 1;
+                                            double eps, int64_t ring, int64_t* report) {
+  if (ring < 0 || !report || !(eps > 0)) return 1;
   SchedStats st;
-  report[11] = 0;
-  const int rc = check_hazards(nc, clusters, nb, blocks, rank_cap, tile, nrhs_max, which, -1, ring, report, st);
-  if (rc == 0 || rc == 9) report[11] = st.ring_wraps;
+  report[11] = report[12] = report[13] = report[14] = 0;
+  const int rc = check_hazards(nc, clusters, nb, blocks, rank_cap, tile, nrhs_max, which, -1,
+                               accumulate_updates(tile, eps), ring, report, st, report + 14);
+  if (rc == 0 || rc == 9) {
+    report[11] = st.ring_wraps;
+    report[12] = st.early_pieces;
+    report[13] = st.accumulated;
+  }
   return rc;
 }

@@ -147,6 +147,8 @@ struct SchedStats {
   int64_t n_factor_tasks = 0, n_solve_tasks = 0;
   int64_t temp_elems = 0;
   int64_t ring_wraps = 0;
+  int64_t early_pieces = 0;  // noted updates added before their block was reached, to free their memory
+  bool accumulated = false;  // whether the updates were accumulated
   double host_ms = 0;
 };
 
@@ -156,12 +158,15 @@ struct SchedStats {
 // `tile`: every block-tree node whose row and column clusters both hold at most
 // `tile` DOFs is factored as one dense tile (tile <= leaf keeps the block tree
 // as it is).  factor_blocks (optional) receives the factor tree the schedules
-// and the arena layout refer to.  ring_elems: size of the region for
+// and the arena layout refer to.  accumulate: sums each leaf's updates before
+// truncating them (accumulate_updates).  ring_elems: size of the region for
 // temporaries (0: by the factor's size); throws when it cannot hold them.
 void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& B, int32_t rank_cap,
                      int32_t nrhs_max, int32_t tile, ArenaLayout& L,
                      Schedule& factor, Schedule& solve, SchedStats& st, std::vector<Block>* factor_blocks,
-                     int64_t ring_elems = 0);
+                     bool accumulate, int64_t ring_elems = 0);
+// Whether the library accumulates the updates of a factorisation.
+bool accumulate_updates(int32_t tile, double eps);
 std::vector<Block> factor_tree(const std::vector<Cluster>& C, const std::vector<Block>& B, int32_t tile);
 
 // The Schulz iteration for the inverse of A_H (Sec. 3, Sec. 4) over four

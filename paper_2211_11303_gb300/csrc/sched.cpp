@@ -61,11 +61,10 @@ struct Buf {
   int64_t seg0;
 };
 
-// Pieces per truncation (beside the target itself).  Larger batches truncate
-// less often; smaller ones leave less work to the task that the newest piece
-// completes (n = 24 factorisation: 4 pieces 881 ms, 8 pieces 709 ms, 16 pieces
-// 782 ms).  Without tiles (tile 0: the block tree's own leaves) every
-// update is truncated by itself, step by step as the recursion writes it.
+// Pieces per truncation of accumulated updates (beside the target itself).
+// Larger batches truncate less often; smaller ones leave less work to the task
+// that the newest piece completes (n = 24 factorisation: 4 pieces 881 ms, 8
+// pieces 709 ms, 16 pieces 782 ms).
 constexpr size_t kBatch = 8;
 constexpr size_t kDirect = 4;  // more pieces of a small target are summed densely first
 constexpr size_t kDenseBatch = 16;  // pieces per dense update
@@ -75,14 +74,20 @@ constexpr size_t kDenseBatch = 16;  // pieces per dense update
 // whole); larger ones quadrant by quadrant first.
 constexpr int32_t kOneStepAgglomeration = 128;
 
+// A ring too small for the temporaries that a schedule holds.
+struct RingFull : std::runtime_error {
+  RingFull() : std::runtime_error("temporaries of one block's update exceed the ring") {}
+};
+
 class Sched {
  public:
+  // accumulate: see gemm
   Sched(const std::vector<Cluster>& C, const std::vector<Block>& B, int32_t kcap, ArenaLayout& L,
         Schedule* S, std::vector<int32_t>& dbuf, std::vector<int32_t>& xbuf,
-        std::vector<int32_t>& ybuf, bool make_buffers, int32_t segsz, int32_t tile,
+        std::vector<int32_t>& ybuf, bool make_buffers, int32_t segsz, bool accumulate,
         int64_t ring_off, int64_t ring_size)
       : C_(C), B_(B), kcap_(kcap), L_(L), S_(S), dbuf_(dbuf), xbuf_(xbuf), ybuf_(ybuf),
-        ring_off_(ring_off), ring_size_(ring_size), batch_(tile > 0 ? kBatch : 1) {
+        ring_off_(ring_off), ring_size_(ring_size), accumulate_(accumulate) {
     S_->pred_ptr.assign(1, 0);
     updates_.resize(B_.size());
     // dependency segments: clusters of at most `segsz` DOFs whose parent is
@@ -142,7 +147,7 @@ class Sched {
   int64_t alloc(int64_t n) {
     n = (n + 31) & ~int64_t(31);
     temp_elems_ += n;
-    if (n > ring_size_) throw std::runtime_error("temporary larger than the ring");
+    if (n > ring_size_) throw RingFull();
     add_old_pieces(n);
     if (cursor_ + n > ring_size_) {
       cursor_ = 0;
@@ -204,6 +209,7 @@ class Sched {
         std::sort(old.begin(), old.end(), [](const Update& x, const Update& y) { return x.seq < y.seq; });
         std::vector<PieceMV> ps;
         for (const Update& u : old) ps.push_back(PieceMV{u.p, 0, 0, u.sign});
+        early_pieces_ += (int64_t)ps.size();
         if (!ps.empty()) add_down(c, ps);
       }
     }
@@ -389,7 +395,7 @@ class Sched {
   void note_access(int32_t b) {
     if (acc_last_[b] == cur_) return;
     if (buf_chunk_[b] >= 0 && chunk_pass_[buf_chunk_[b]] != buf_pass_[b])
-      throw std::runtime_error("temporaries of one block's update exceed the ring");
+      throw RingFull();
     acc_last_[b] = cur_;
     grow4(acc_task_);
     grow4(acc_next_);
@@ -696,7 +702,9 @@ class Sched {
   }
   // Ends of the batches of n pieces, oldest first: the short one comes first
   // (ending with one or two pieces, n = 24 took 837 ms instead of 709 ms).
-  static std::vector<size_t> batches(size_t n, size_t most) {
+  // Updates that are not accumulated are truncated whole.
+  std::vector<size_t> batches(size_t n) const {
+    const size_t most = accumulate_ ? kBatch : std::max<size_t>(n, 1);
     std::vector<size_t> ends;
     for (size_t q = n % most ? n % most : most; q < n; q += most) ends.push_back(q);
     ends.push_back(n);
@@ -765,11 +773,11 @@ class Sched {
     r.Y.buf = new_buf_leaves(cc);
     bind_alloc(r.Y.buf);
     r.Y.v = View{yo, 1, sz(cc), sz(cc), cap, slot, 0};
-    if (batch_ > 1 && small_target(rc, cc) && ps.size() > kDirect) {
+    if (accumulate_ && small_target(rc, cc) && ps.size() > kDirect) {
       emit_trunc(r.X, r.Y, slot, cap, {dense_sum(rc, cc, ps)});
       return r;
     }
-    const std::vector<size_t> ends = batches(ps.size(), batch_);
+    const std::vector<size_t> ends = batches(ps.size());
     for (size_t k = 0, q0 = 0; k < ends.size(); q0 = ends[k++]) {
       std::vector<PieceMV> batch;
       if (q0 > 0) batch.push_back(PieceMV{r, 0, 0, 1.0f});
@@ -812,6 +820,29 @@ class Sched {
     if (ka == KIND_DENSE) return LR{mvIdent(tau), hmul_new(b, mvDT(a), true)};
     return LR{hmul_new(a, mvD(b), false), mvIdent(rho)};
   }
+  // X Y^T = the product of any two blocks, two subdivided ones agglomerated:
+  // the eight son products in one truncation for a small target, else two per
+  // quadrant (four independent tasks) and then the four quadrants.
+  LR product_any(int32_t a, int32_t b) {
+    if (!both_sub(a, b)) return product(a, b);
+    const Cluster& T = C_[rowc(a)];
+    const Cluster& R = C_[colc(b)];
+    const bool one_step = small_target(rowc(a), colc(b));
+    std::vector<PieceMV> ps;
+    for (int i = 0; i < 2; ++i)
+      for (int j = 0; j < 2; ++j) {
+        const int32_t ts = T.son[i], rs = R.son[j], xo = C_[ts].off - T.off, yo = C_[rs].off - R.off;
+        std::vector<PieceMV> q;
+        for (int k = 0; k < 2; ++k) q.push_back(PieceMV{product_any(son(a, i, k), son(b, k, j)), 0, 0, 1.0f});
+        if (!one_step) q = {PieceMV{trunc_new(ts, rs, q), 0, 0, 1.0f}};
+        for (PieceMV& p : q) {
+          p.xoff = xo;
+          p.yoff = yo;
+          ps.push_back(p);
+        }
+      }
+    return trunc_new(rowc(a), colc(b), ps);
+  }
   bool both_sub(int32_t a, int32_t b) const { return kind(a) == KIND_SUB && kind(b) == KIND_SUB; }
   typedef std::vector<std::pair<int32_t, int32_t>> Pairs;
 
@@ -831,7 +862,7 @@ class Sched {
     if (subs.empty()) return;
     const Cluster& T = C_[tau];
     const Cluster& R = C_[rho];
-    const bool one_step = T.size <= kOneStepAgglomeration && R.size <= kOneStepAgglomeration;
+    const bool one_step = small_target(tau, rho);
     for (int i = 0; i < 2; ++i)
       for (int j = 0; j < 2; ++j) {
         const int32_t ts = T.son[i], rs = R.son[j], xo = xoff + C_[ts].off - T.off, yo = yoff + C_[rs].off - R.off;
@@ -848,8 +879,7 @@ class Sched {
       }
   }
 
-  // c <- c + sign * sum_p X_p Y_p^T in the format of c, batch_ pieces per
-  // truncation of a low-rank c (per task of a dense one)
+  // c <- c + sign * sum_p X_p Y_p^T in the format of c, a leaf, in batches
   // (sums: small targets may sum many pieces densely first, which allocates)
   void add_pieces(int32_t c, const std::vector<PieceMV>& ps, bool sums = true) {
     if (kind(c) == KIND_DENSE) {
@@ -866,13 +896,13 @@ class Sched {
       }
       return;
     }
-    if (sums && batch_ > 1 && small_target(rowc(c), colc(c)) && ps.size() > kDirect) {
+    if (sums && accumulate_ && small_target(rowc(c), colc(c)) && ps.size() > kDirect) {
       const PieceMV sum = dense_sum(rowc(c), colc(c), ps);
       emit_trunc(mvX(c), mvY(c), L_.slot[c], L_.cap[c], {PieceMV{LR{mvX(c), mvY(c)}, 0, 0, 1.0f}, sum});
       return;
     }
     if (ps.empty()) return;
-    const std::vector<size_t> ends = batches(ps.size(), batch_);
+    const std::vector<size_t> ends = batches(ps.size());
     for (size_t k = 0, q0 = 0; k < ends.size(); q0 = ends[k++]) {
       std::vector<PieceMV> batch;
       batch.push_back(PieceMV{LR{mvX(c), mvY(c)}, 0, 0, 1.0f});
@@ -882,17 +912,49 @@ class Sched {
   }
 
   // c <- c + sign * a b in the format of c (the H-LU's Schur complement update
-  // is sign = -1), accumulated: the update is noted at c and moves down the
-  // block tree when c is used (settle), so that a leaf receives the updates of
-  // all steps and levels together and truncates their sum.  Eager updates
-  // truncated every leaf once per step: 1.14 M truncations and 4.7 M dense
-  // updates at n = 24, 0.19 M and 0.70 M accumulated.
+  // is sign = -1).
+  // Accumulated: the update is noted at c and moves down the block tree when c
+  // is used (settle), so that a leaf receives the updates of all steps and
+  // levels together and truncates their sum in batches.  At n = 24 that is 0.19
+  // M truncations and 0.70 M dense updates instead of 1.14 M and 4.7 M.
+  // Otherwise every product is formed at the largest block it has and added at
+  // once, down to the leaves, each of which truncates it.
   void gemm(int32_t c, int32_t a, int32_t b, float sign = -1.0f) {
+    if (!accumulate_) {
+      gemm_at_once(c, a, b, sign);
+      return;
+    }
     Update u;
     u.a = a;
     u.b = b;
     u.sign = sign;
     note_update(c, u);
+  }
+  void gemm_at_once(int32_t c, int32_t a, int32_t b, float sign) {
+    if (kind(c) != KIND_SUB || !both_sub(a, b)) {
+      add_products(c, {product_any(a, b)}, sign);
+      return;
+    }
+    for (int i = 0; i < 2; ++i)
+      for (int j = 0; j < 2; ++j) {
+        // the two son products into c_ij that are not themselves subdivided
+        // products are added together
+        const int32_t cc = son(c, i, j);
+        std::vector<LR> ps;
+        for (int k = 0; k < 2; ++k) {
+          const int32_t aa = son(a, i, k), bb = son(b, k, j);
+          if (kind(cc) == KIND_SUB && both_sub(aa, bb))
+            gemm_at_once(cc, aa, bb, sign);
+          else
+            ps.push_back(product_any(aa, bb));
+        }
+        add_products(cc, ps, sign);
+      }
+  }
+  void add_products(int32_t c, const std::vector<LR>& ps, float sign) {
+    std::vector<PieceMV> pieces;
+    for (const LR& p : ps) pieces.push_back(PieceMV{p, 0, 0, sign});
+    if (!pieces.empty()) add_down(c, pieces);
   }
   // The updates noted at c, before c is factored, solved or read: a leaf adds
   // them, a subdivided block hands them to its sons (products that are not
@@ -1246,7 +1308,7 @@ class Sched {
   int32_t seg_size_of(int32_t) const { return segsz_; }
   int32_t segsz_ = 0;
   int64_t ring_off_ = 0, ring_size_ = 0, cursor_ = 0;
-  size_t batch_;  // pieces per truncation
+  bool accumulate_;
   std::vector<int32_t> seg_begin_, seg_end_, seg_cluster_;
   std::vector<std::vector<int32_t>> chunk_occ_;
   std::vector<int32_t> chunk_fence_task_;
@@ -1254,6 +1316,7 @@ class Sched {
   int32_t pass_ = 0;
  public:
   int64_t wraps_ = 0;
+  int64_t early_pieces_ = 0;  // pieces that add_old_pieces added
  private:
   std::vector<std::vector<Update>> updates_;                     // per block
   std::unordered_map<int64_t, std::vector<int32_t>> held_;        // per ring bucket: blocks with updates there
@@ -1468,12 +1531,39 @@ void order_for_tickets(Schedule& S) {
   S.pred_idx.swap(pi);
 }
 
+// Builds a schedule with accumulated updates when asked for and, where their
+// temporaries exceed the ring, without.
+template <class F>
+void with_ring(bool accumulate, ArenaLayout& L, const F& build) {
+  if (accumulate) {
+    const ArenaLayout before = L;
+    try {
+      build(true);
+      return;
+    } catch (const RingFull&) {
+      L = before;
+    }
+  }
+  build(false);
+}
+
 }  // namespace
+
+// Without tiles (tile 0: the block tree's own small leaves) the accumulated
+// updates of a leaf are many and make one long chain of truncations: n = 10,
+// leaf 16: 517 ms against 63 ms added at once (FP64, n = 8: 1,838 against 118
+// ms).  With tiles the two take about the same time at eps 1e-3 to 1e-5 (n =
+// 24, FP32, eps 1e-4: 713 against 710 ms), and the accumulated factor is the
+// nearer one (one apply leaves 2e-3 of the residual against 1e-2, n = 24).  At
+// finer eps the sums' spectra are filled with rounding and the wide truncations
+// cost more: n = 16, FP32: 1e-6 374 against 267 ms, 1e-7 697 against 453 ms; n =
+// 11, FP64, 1e-10: 529 against 474 ms.
+bool accumulate_updates(int32_t tile, double eps) { return tile > 0 && eps >= 4e-6; }
 
 void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bfull, int32_t rank_cap,
                      int32_t nrhs_max, int32_t tile, ArenaLayout& L,
                      Schedule& factor, Schedule& solve,
-                     SchedStats& st, std::vector<Block>* factor_blocks, int64_t ring_elems) {
+                     SchedStats& st, std::vector<Block>* factor_blocks, bool accumulate, int64_t ring_elems) {
   std::vector<Block> Bt = factor_tree(C, Bfull, tile);
   const std::vector<Block>& B = Bt;
   if (factor_blocks) *factor_blocks = Bt;
@@ -1543,17 +1633,22 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bf
   factor = Schedule();
   solve = Schedule();
   std::vector<int32_t> dbuf, xbuf, ybuf;
-  {
-    Sched s(C, B, rank_cap, L, &factor, dbuf, xbuf, ybuf, true, segsz, tile, ring_off, ring);
+  // accumulated updates hold factors for longer; where the ring is too small
+  // for that, they are added at once
+  with_ring(accumulate, L, [&](bool acc) {
+    factor = Schedule();
+    Sched s(C, B, rank_cap, L, &factor, dbuf, xbuf, ybuf, true, segsz, acc, ring_off, ring);
     s.lu(0);
     st.temp_elems = s.temp_elems_;
     st.ring_wraps = s.wraps_;
-  }
+    st.early_pieces = s.early_pieces_;
+    st.accumulated = acc;
+  });
   {
     // the solve's units are the leaf clusters, half a tile or so each: a step of
     // the chain spreads over twice as many SMs (n = 24, 8 columns: 8.4 -> 7.8 ms an
     // apply, FP64 n = 11 5.2 -> 3.5 ms)
-    Sched s(C, B, rank_cap, L, &solve, dbuf, xbuf, ybuf, true, leafmax, tile, ring_off, ring);
+    Sched s(C, B, rank_cap, L, &solve, dbuf, xbuf, ybuf, true, leafmax, false, ring_off, ring);
     s.solve_all(nrhs_max);
     st.temp_elems += s.temp_elems_;
   }
@@ -1630,11 +1725,13 @@ void build_inverse_schedules(const std::vector<Cluster>& C, const std::vector<Bl
   std::vector<int32_t> dbuf, xbuf, ybuf;
   const int32_t A0 = 0, X0 = nb, T0 = 2 * nb, Y0 = 3 * nb;
   {
-    Sched s(C, Bx, rank_cap, L, &start, dbuf, xbuf, ybuf, true, segsz, tile, L.ring_off, ring);
+    Sched s(C, Bx, rank_cap, L, &start, dbuf, xbuf, ybuf, true, segsz, false, L.ring_off, ring);
     s.copy_scaled(X0, A0, 1.0f, true);
   }
-  {
-    Sched s(C, Bx, rank_cap, L, &iter, dbuf, xbuf, ybuf, true, segsz, tile, L.ring_off, ring);
+  // (n = 6, FP64, eps 1e-8, twenty steps: 1.7 s accumulated, 8.1 s not)
+  with_ring(tile > 0, L, [&](bool acc) {
+    iter = Schedule();
+    Sched s(C, Bx, rank_cap, L, &iter, dbuf, xbuf, ybuf, true, segsz, acc, L.ring_off, ring);
     s.zero(T0);
     s.gemm(T0, A0, X0, -1.0f);  // T = -A X
     s.settle_all(T0);
@@ -1644,9 +1741,11 @@ void build_inverse_schedules(const std::vector<Cluster>& C, const std::vector<Bl
     s.copy_scaled(X0, Y0, 1.0f, false);
     st.temp_elems = s.temp_elems_;
     st.ring_wraps = s.wraps_;
-  }
+    st.early_pieces = s.early_pieces_;
+    st.accumulated = acc;
+  });
   {
-    Sched s(C, Bx, rank_cap, L, &apply, dbuf, xbuf, ybuf, true, segsz, tile, L.ring_off, ring);
+    Sched s(C, Bx, rank_cap, L, &apply, dbuf, xbuf, ybuf, true, segsz, false, L.ring_off, ring);
     const int32_t N = C[0].size;
     MV Win, Wout;
     Win.buf = -1;  // read-only here
