@@ -1687,7 +1687,6 @@ __device__ bool task_trunc_dense(Ctx<T>& c, const Task& t, char* smem) {
     t0 = t1;
   }
   if (rp == kDenseRank && tail2 > T(c.eps * c.eps) * piv2) {
-    if (threadIdx.x == 0) atomicAdd(c.status + 5, 1);
     __syncthreads();
     return false;
   }
@@ -2415,10 +2414,7 @@ __device__ bool task_trunc_sampled(Ctx<T>& c, const Task& t, char* smem, int W) 
     // (sm.inv holds 1 / pivot norm)
     const T miss = tail * T(k) / (f2 * first * T(k - rp));  // (missed / 0.1 eps s_1)^2
     const bool flat = rp >= 16 && sm.inv[rp - 9] >= T(0.5) * sm.inv[rp - 1];
-    if (!(miss <= T(sizeof(T) == 4 ? 30 : 1) || (sizeof(T) == 4 && flat && miss <= T(100)))) {
-      if (threadIdx.x == 0) atomicAdd(c.status + 5, 1);
-      return false;
-    }
+    if (!(miss <= T(sizeof(T) == 4 ? 30 : 1) || (sizeof(T) == 4 && flat && miss <= T(100)))) return false;
   }
   if (rp == 0) {
     __syncthreads();
@@ -2504,13 +2500,19 @@ __device__ void task_trunc(Ctx<T>& c, const Task& t, char* smem) {
     if (threadIdx.x == 0) __stcg(c.ranks + t.out_slot, 0);
     return;
   }
-  if (m <= kDenseMax && n <= kDenseMax && task_trunc_dense(c, t, smem)) return;
+  bool redone = false;
+  if (m <= kDenseMax && n <= kDenseMax) {
+    if (task_trunc_dense(c, t, smem)) return;
+    redone = true;
+  }
   // below kRsEps the rounding of the samples is above eps
   constexpr double kRsEps = sizeof(T) == 4 ? 5e-7 : 1e-13;
-  if (wsum > kRsMin && wsum <= kRsCols && t.list_count <= kRsPieces && min(m, n) >= 64 && c.eps >= kRsEps &&
-      task_trunc_sampled(c, t, smem, wsum))
-    return;
+  if (wsum > kRsMin && wsum <= kRsCols && t.list_count <= kRsPieces && min(m, n) >= 64 && c.eps >= kRsEps) {
+    if (task_trunc_sampled(c, t, smem, wsum)) return;
+    redone = true;
+  }
   __syncthreads();
+  if (redone && threadIdx.x == 0) atomicAdd(c.status + 5, 1);
   // the whole stack in shared memory, one compression
   if (trunc_small_fits<T>(m, n, wsum)) {
     task_trunc_small(c, t, smem, wsum);
