@@ -1919,10 +1919,16 @@ __device__ void task_trunc_small(Ctx<T>& c, const Task& t, char* smem, int W) {
 // The samples that the pivots leave over estimate what Q misses: their mean
 // square is ||A - Q Q^T A||_F^2, and the first pivot's share of all samples'
 // energy times ||A||_F^2 is at most s_1^2.  The steps stop once the one is
-// below (0.1 eps)^2 of the other.  In FP32, at the end (6 samples left over,
-// or 64 columns kept) (0.55 eps)^2 will do, or eps^2 when the last nine pivots are level: what is missed is then
-// spread over many directions (the rounding of cancelling pieces), each far
-// below the Frobenius norm.  Otherwise, or when a Gram matrix is numerically
+// below (0.1 eps)^2 of the other (in FP32 no finer than five units of the
+// samples' rounding, 0.3 eps at eps 1e-6).  In FP32, at the end (6 samples left
+// over, or 64 columns kept) (0.55 eps)^2 will do, or eps^2 when the last nine
+// pivots are level: what is missed is then spread over many directions (the
+// rounding of cancelling pieces), each far below the Frobenius norm.  The other
+// routes stop at 0.1 eps: where a shelf of values lies at 0.05 eps the error is
+// 0.11 eps instead of 0.05 eps (300 x 257, 80 columns); the factor is no worse
+// for it (one apply leaves 2e-3 of the residual at n = 24, eps 1e-4, the stack
+// route for every one of these targets 7e-3, and takes 838 instead of 713 ms).
+// Otherwise, or when a Gram matrix is numerically
 // singular, the task falls back to the stack route (nothing has been written yet).
 // Q and P are orthonormalised once more by their Gram matrices: the
 // Gram-Schmidt vectors of small pivots are only as orthogonal as the pivots' range.
@@ -2401,8 +2407,7 @@ __device__ bool task_trunc_sampled(Ctx<T>& c, const Task& t, char* smem, int W) 
   expand(xat, sm.xlo, sm.xhi, m, k, S);
   lap(0);
   const T f2 = T(0.01 * c.eps * c.eps);
-  // the steps also end at the rounding of the samples, five units (FP32 at
-  // eps 1e-6: 0.3 eps); beyond it the pivots are noise
+  // the steps also end at the rounding of the samples; beyond it the pivots are noise
   const T noise = sizeof(T) == 4 ? T(9e-14) : T(3e-31);
   const T floor2 = max(f2, noise);
   T tail = 0, first = 0;
@@ -2505,8 +2510,10 @@ __device__ void task_trunc(Ctx<T>& c, const Task& t, char* smem) {
     if (task_trunc_dense(c, t, smem)) return;
     redone = true;
   }
-  // below kRsEps the rounding of the samples is above eps
-  constexpr double kRsEps = sizeof(T) == 4 ? 5e-7 : 1e-13;
+  // below kRsEps the samples' rounding floor comes close to eps (FP32, 150 x 140,
+  // 30 columns, values left at 0.05 eps: at 5e-7 an error of 1.1 eps, from the
+  // stack 0.5 eps; at 1e-6 the two are alike)
+  constexpr double kRsEps = sizeof(T) == 4 ? 1e-6 : 1e-13;
   if (wsum > kRsMin && wsum <= kRsCols && t.list_count <= kRsPieces && min(m, n) >= 64 && c.eps >= kRsEps) {
     if (task_trunc_sampled(c, t, smem, wsum)) return;
     redone = true;
