@@ -307,7 +307,6 @@ struct hlu_handle {
   int32_t* d_ranks = nullptr;
   int32_t cur_nrhs = 0;  // the value last written to the right-hand-side count slot
   int32_t* d_term_p = nullptr;  // solve terms' column counts after the last factorisation
-  bool term_p_fresh = false;
   int32_t* d_piv = nullptr;
   void* d_scratch = nullptr;
   int64_t scratch_stride = 0;
@@ -336,7 +335,6 @@ void free_factor(hlu_handle* h) {
                   (void*)h->d_prof})
     if (p) dev_free(p);
   h->d_prof = nullptr;
-  h->term_p_fresh = false;
   h->d_arena = nullptr;
   h->d_ranks = nullptr;
   h->d_piv = nullptr;
@@ -370,18 +368,6 @@ __global__ void k_term_ranks(const Term* terms, int64_t n, const int32_t* ranks,
   }
 }
 
-// The term widths of h's triangular solve, resolved before the first solve
-// after a factorisation (stream-ordered after the ranks it produced).
-int prepare_terms(hlu_handle* h, cudaStream_t s) {
-  if (h->dS.nterms == 0 || h->term_p_fresh) return HLU_OK;
-  const int blocks = (int)std::min<int64_t>((h->dS.nterms + 255) / 256, 1184);
-  note_launch();
-  k_term_ranks<<<blocks, 256, 0, s>>>(h->dS.terms, h->dS.nterms, h->d_ranks, h->L.nrhs_slot, h->d_term_p);
-  CKR(cudaGetLastError(), "term widths");
-  h->term_p_fresh = true;
-  return HLU_OK;
-}
-
 // One launch of the triangular solves of several handles with the same
 // precision, on the columns in their work vectors.  Handle 0's status is used.
 int solve_run(hlu_handle* const* hs, int count, cudaStream_t s) {
@@ -393,7 +379,6 @@ int solve_run(hlu_handle* const* hs, int count, cudaStream_t s) {
     if (h->precision != hs[0]->precision) return fail(HLU_ERR_ARG, "mixed precisions in a batch");
     for (int j = 0; j < i; ++j)
       if (hs[j] == h) return fail(HLU_ERR_ARG, "a handle appears twice in a batch");
-    if (int rc = prepare_terms(h, s)) return rc;
     SolveProb& p = a.probs[i];
     p.tasks = h->dS.tasks;
     p.terms = h->dS.terms;
@@ -1196,7 +1181,6 @@ static int factor_prepare(hlu_handle* h, int32_t precision, cudaStream_t s) {
     CKR(dev_malloc(&h->d_prof, sizeof(unsigned long long) * kProfEntries), "prof");
   }
   h->precision = precision;
-  h->term_p_fresh = false;
   CKR(cudaMemsetAsync(h->d_ranks, 0, sizeof(int32_t) * std::max(h->L.n_slots, 1), s), "ranks");
   h->cur_nrhs = 0;
   int32_t st0[8] = {0, -1, 0, 0, 0, 0, 0, 0};
@@ -1219,9 +1203,17 @@ static int factor_prepare(hlu_handle* h, int32_t precision, cudaStream_t s) {
   return HLU_OK;
 }
 
-// after a factorisation was launched: the solve blocks' inverses (status_of:
-// the handle whose status words the launch uses)
-static int factor_inverses(hlu_handle* h, const hlu_handle* status_of, cudaStream_t s) {
+// Queued behind a factorisation: what the triangular solve reads beside the
+// factor, its terms' widths and (of a whole factorisation) the solve blocks'
+// inverses.  status_of: the handle whose status words the launch uses.
+static int factor_solve_data(hlu_handle* h, const hlu_handle* status_of, bool whole, cudaStream_t s) {
+  if (h->dS.nterms > 0) {
+    const int blocks = (int)std::min<int64_t>((h->dS.nterms + 255) / 256, 1184);
+    note_launch();
+    k_term_ranks<<<blocks, 256, 0, s>>>(h->dS.terms, h->dS.nterms, h->d_ranks, h->L.nrhs_slot, h->d_term_p);
+    CKR(cudaGetLastError(), "term widths");
+  }
+  if (!whole) return HLU_OK;
   const SchedBundle& b = *h->sb;
   const int32_t nu = (int32_t)b.L.inv_units.size(), nl = (int32_t)b.L.inv_leaves.size();
   if (h->precision == HLU_FP64)
@@ -1285,7 +1277,7 @@ static int factor_impl(hlu_handle* h, int32_t precision, void* stream, int64_t l
     CKR(cudaEventRecord(h->ev0, s), "event");
     rc = exec_run(h, h->dF, h->grid, s, true, limit);
     if (rc) return rc;
-    if (limit < 0 && (rc = factor_inverses(h, h, s))) return rc;
+    if ((rc = factor_solve_data(h, h, limit < 0, s))) return rc;
     CKR(cudaEventRecord(h->ev1, s), "event");
     CKR(cudaEventSynchronize(h->ev1), "sync");
     float ms = 0;
@@ -1310,7 +1302,7 @@ int hlu_factor_async(hlu_handle* h, int32_t precision, int32_t max_ctas, void* s
     const int grid = max_ctas > 0 ? std::min(h->grid, (int)max_ctas) : h->grid;
     rc = exec_run(h, h->dF, grid, s, true);
     if (rc) return rc;
-    if ((rc = factor_inverses(h, h, s))) return rc;
+    if ((rc = factor_solve_data(h, h, true, s))) return rc;
     CKR(cudaEventRecord(h->ev1, s), "event");
     h->factor_pending = true;
     h->factor_stream = s;
@@ -1701,7 +1693,7 @@ int hlu_factor_batch(hlu_handle** hs, int32_t count, int32_t precision, void* st
     int rc = exec_run_batch(hs, count, s, &g_batch_q, &g_batch_q_len);
     if (rc) return rc;
     for (int32_t i = 0; i < count; ++i)
-      if ((rc = factor_inverses(hs[i], hs[0], s))) return rc;
+      if ((rc = factor_solve_data(hs[i], hs[0], true, s))) return rc;
     CKR(cudaEventRecord(hs[0]->ev1, s), "event");
     CKR(cudaEventSynchronize(hs[0]->ev1), "sync");
     float ms = 0;

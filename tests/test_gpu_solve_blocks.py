@@ -66,3 +66,41 @@ def test_bounded_wait_of_the_solve_reports_a_timeout(hlu):
         assert hlu.gmres_solve(h, b, x, tol=1e-10)["converged"] == 1
     finally:
         hlu.hlu_destroy(h)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_first_solve_of_a_factor_under_capture(hlu, prec):
+    """hlu_solve captured in a graph before any other solve of the factor: what
+    the solve reads beside the factor belongs to the factorisation, so eager
+    solves and replays before and after another factorisation agree."""
+    P = hlu.HLU_FP64 if prec == "fp64" else hlu.HLU_FP32
+    other = hlu.hlu_build(4, 2.0, 16, 2.0, 1e-4)
+    h = hlu.hlu_build(6, 3.0, 16, 2.0, 1e-4)
+    try:
+        N = hlu.hlu_n(h)
+        b = hlu.colmajor(N, 3)
+        b.copy_(torch.from_numpy(np.stack([synth.normal(70 + j, N) for j in range(3)], axis=1)))
+        x, y = hlu.colmajor(N, 3), hlu.colmajor(N, 3)
+        hlu.hlu_factor(other, P)  # loads the solve's kernels
+        no = hlu.hlu_n(other)
+        hlu.hlu_solve(other, torch.ones(no, dtype=torch.float64, device="cuda"),
+                      torch.empty(no, dtype=torch.float64, device="cuda"))
+        hlu.hlu_factor(h, P)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            hlu.hlu_solve(h, b, x)
+        hlu.hlu_solve(h, b, y)  # eager, before the first replay
+        r = torch.empty_like(y)
+        hlu.hlu_spmv(h, y, r)
+        assert (torch.linalg.norm(r - b) / torch.linalg.norm(b)).item() < 0.1
+        for again in (False, True):
+            if again:
+                hlu.hlu_factor(h, P)
+            x.zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(x, y)
+    finally:
+        hlu.hlu_destroy(h)
+        hlu.hlu_destroy(other)
