@@ -1645,10 +1645,12 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bf
     st.accumulated = acc;
   });
   {
-    // the solve's units are the leaf clusters, half a tile or so each: a step of
-    // the chain spreads over twice as many SMs (n = 24, 8 columns: 8.4 -> 7.8 ms an
-    // apply, FP64 n = 11 5.2 -> 3.5 ms)
-    Sched s(C, B, rank_cap, L, &solve, dbuf, xbuf, ybuf, true, leafmax, false, ring_off, ring);
+    // the solve's units are clusters of half a tile: a step of the chain spreads
+    // over twice as many SMs as with whole ones (n = 24, 8 columns: 8.4 -> 7.8 ms
+    // an apply, FP64 n = 11 5.2 -> 3.5 ms).  Smaller leaves are no units of their
+    // own: their edges are many (n = 16: 0.27 M with units of 32, 2.4 M with leaves
+    // of 8, 27 M with leaves of 2) and their rows leave lanes idle.
+    Sched s(C, B, rank_cap, L, &solve, dbuf, xbuf, ybuf, true, std::max(leafmax, tile / 2), false, ring_off, ring);
     s.solve_all(nrhs_max);
     st.temp_elems += s.temp_elems_;
   }
