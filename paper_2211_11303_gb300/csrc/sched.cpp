@@ -12,11 +12,14 @@
 //
 // Ranks of low-rank blocks are data dependent.  The schedule only uses rank
 // capacities; kernels read the live rank from a rank slot when they run.
+#include <sys/mman.h>
+
 #include <algorithm>
 #include <chrono>
 #include <cstdlib>
 #include <cstring>
 #include <functional>
+#include <future>
 #include <queue>
 #include <stdexcept>
 #include <unordered_map>
@@ -31,11 +34,18 @@ namespace {
 // terms, 0.9 GB of predecessor indices), and every reallocation writes its
 // new block once.  Growing by 4 instead of 2 writes about 4/3 of the final
 // size instead of about 2x, which took a quarter off the n = 24 build (most
-// of it page faults); the unused capacity is address space only.
+// of it page faults); the unused capacity is address space only.  Blocks of
+// some megabytes ask for huge pages where the system gives them on request.
 template <class V>
 inline void grow4(V& v, size_t extra = 1) {
-  if (v.size() + extra > v.capacity())
-    v.reserve(std::max<size_t>(v.size() + extra, std::max<size_t>(4096, v.capacity() * 4)));
+  if (v.size() + extra <= v.capacity()) return;
+  v.reserve(std::max<size_t>(v.size() + extra, std::max<size_t>(4096, v.capacity() * 4)));
+#ifdef MADV_HUGEPAGE
+  constexpr uintptr_t kHuge = uintptr_t(1) << 21;
+  const uintptr_t lo = ((uintptr_t)(v.data() + v.size()) + kHuge - 1) & ~(kHuge - 1);
+  const uintptr_t hi = (uintptr_t)(v.data() + v.capacity()) & ~(kHuge - 1);
+  if (hi > lo) madvise((void*)lo, hi - lo, MADV_HUGEPAGE);
+#endif
 }
 
 constexpr int64_t kNotTemp = INT64_MAX;
@@ -52,13 +62,25 @@ struct PieceMV {
   LR p;
   int32_t xoff, yoff;
   float sign;
-  std::vector<int32_t> windows;  // a dense sum: the dependency buffers of its windows
+  int32_t win0 = 0, nwin = 0;  // a dense sum: the dependency buffers of its windows
 };
 
+// A dependency buffer: its segments, the tasks that touched it, and of a
+// temporary the fences of its memory and where that lies in the ring.
 struct Buf {
   int32_t base_leaf;
   int32_t nseg;
   int64_t seg0;
+  int64_t acc_head = -1;   // list of accesses (acc_task_, acc_next_)
+  int64_t fence_begin = 0;  // fences in fence_pool_
+  int32_t n_fences = 0;
+  int32_t acc_last = -1;    // the last task on the list
+  int32_t chunk = -1, pass = 0;  // a temporary's first chunk (else -1) and its pass
+};
+struct Seg {
+  int32_t writer = -1;
+  int32_t buf = -1;
+  int64_t rhead = -1;  // readers since (rtask_, rnext_)
 };
 
 // Pieces per truncation of accumulated updates (beside the target itself).
@@ -170,7 +192,7 @@ class Sched {
           saved_deps.swap(deps_);
           begin(f);
           for (int32_t old : chunk_occ_[ch])
-            for (int64_t r = acc_head_[old]; r >= 0; r = acc_next_[r]) dep(acc_task_[r]);
+            for (int64_t r = bufs_[old].acc_head; r >= 0; r = acc_next_[r]) dep(acc_task_[r]);
           end();
           chunk_fence_task_[ch] = cur_;
           deps_.swap(saved_deps);
@@ -250,50 +272,36 @@ class Sched {
     if (!pending_fence_.empty()) {
       std::sort(pending_fence_.begin(), pending_fence_.end());
       pending_fence_.erase(std::unique(pending_fence_.begin(), pending_fence_.end()), pending_fence_.end());
-      fence_begin_[b] = (int64_t)fence_pool_.size();
+      bufs_[b].fence_begin = (int64_t)fence_pool_.size();
+      bufs_[b].n_fences = (int32_t)pending_fence_.size();
       fence_pool_.insert(fence_pool_.end(), pending_fence_.begin(), pending_fence_.end());
-      fence_end_[b] = (int64_t)fence_pool_.size();
       pending_fence_.clear();
     }
     for (int64_t ch = last_alloc_lo_; ch <= last_alloc_hi_; ++ch) chunk_occ_[ch].push_back(b);
-    buf_chunk_[b] = (int32_t)last_alloc_lo_;
-    buf_pass_[b] = pass_;
+    bufs_[b].chunk = (int32_t)last_alloc_lo_;
+    bufs_[b].pass = pass_;
   }
   int32_t new_slot() { return L_.n_slots++; }
   int64_t temp_elems_ = 0;
   int64_t peak_ = 0;
 
   // ---------------------------------------------------------------- buffers
-  int32_t push_buf(const Buf& b) {
+  int32_t push_buf(int32_t base_leaf, int32_t nseg) {
+    const int32_t id = (int32_t)bufs_.size();
+    Buf b;
+    b.base_leaf = base_leaf;
+    b.nseg = nseg;
+    b.seg0 = (int64_t)segs_.size();
+    Seg g;
+    g.buf = id;
+    grow4(segs_, nseg);
+    segs_.resize(segs_.size() + nseg, g);
+    grow4(bufs_);
     bufs_.push_back(b);
-    acc_head_.push_back(-1);
-    acc_last_.push_back(-1);
-    buf_chunk_.push_back(-1);
-    buf_pass_.push_back(0);
-    fence_begin_.push_back(0);
-    fence_end_.push_back(0);
-    return (int32_t)bufs_.size() - 1;
+    return id;
   }
-  int32_t new_buf_leaves(int32_t clus) {
-    Buf b;
-    b.base_leaf = seg_begin_[clus];
-    b.nseg = seg_end_[clus] - seg_begin_[clus];
-    b.seg0 = (int64_t)seg_writer_.size();
-    seg_writer_.resize(seg_writer_.size() + b.nseg, -1);
-    seg_rhead_.resize(seg_rhead_.size() + b.nseg, -1);
-    seg_buf_.resize(seg_buf_.size() + b.nseg, (int32_t)bufs_.size());
-    return push_buf(b);
-  }
-  int32_t new_buf_single() {
-    Buf b;
-    b.base_leaf = -1;
-    b.nseg = 1;
-    b.seg0 = (int64_t)seg_writer_.size();
-    seg_writer_.push_back(-1);
-    seg_rhead_.push_back(-1);
-    seg_buf_.push_back((int32_t)bufs_.size());
-    return push_buf(b);
-  }
+  int32_t new_buf_leaves(int32_t clus) { return push_buf(seg_begin_[clus], seg_end_[clus] - seg_begin_[clus]); }
+  int32_t new_buf_single() { return push_buf(-1, 1); }
 
   // ---------------------------------------------------------------- views
   int32_t rowc(int32_t b) const { return B_[b].row; }
@@ -376,6 +384,8 @@ class Sched {
   int32_t begin(const Task& t) {
     int32_t id = (int32_t)S_->tasks.size();
     grow4(S_->tasks);
+    grow4(stamp_);
+    grow4(implied_);
     S_->tasks.push_back(t);
     stamp_.push_back(-1);
     implied_.push_back(-1);
@@ -392,33 +402,34 @@ class Sched {
   // A temporary may be used until its first chunk is entered in a later pass of
   // the ring: the fence made then orders the chunk's next occupants after the
   // accesses noted so far, and no later one.
-  void note_access(int32_t b) {
-    if (acc_last_[b] == cur_) return;
-    if (buf_chunk_[b] >= 0 && chunk_pass_[buf_chunk_[b]] != buf_pass_[b])
-      throw RingFull();
-    acc_last_[b] = cur_;
+  void note_access(int32_t id) {
+    Buf& b = bufs_[id];
+    if (b.acc_last == cur_) return;
+    if (b.chunk >= 0 && chunk_pass_[b.chunk] != b.pass) throw RingFull();
+    b.acc_last = cur_;
     grow4(acc_task_);
     grow4(acc_next_);
     acc_task_.push_back(cur_);
-    acc_next_.push_back(acc_head_[b]);
-    acc_head_[b] = (int64_t)acc_task_.size() - 1;
+    acc_next_.push_back(b.acc_head);
+    b.acc_head = (int64_t)acc_task_.size() - 1;
   }
   void touch(int64_t seg, bool w) {
-    const int32_t b = seg_buf_[seg];
-    if (seg_writer_[seg] < 0)
-      for (int64_t f = fence_begin_[b]; f < fence_end_[b]; ++f) dep(fence_pool_[f]);
-    note_access(b);
-    dep(seg_writer_[seg]);
+    Seg& g = segs_[seg];
+    const Buf& b = bufs_[g.buf];
+    if (g.writer < 0)
+      for (int64_t f = b.fence_begin; f < b.fence_begin + b.n_fences; ++f) dep(fence_pool_[f]);
+    note_access(g.buf);
+    dep(g.writer);
     if (w) {
-      for (int64_t r = seg_rhead_[seg]; r >= 0; r = rnext_[r]) dep(rtask_[r]);
-      seg_rhead_[seg] = -1;
-      seg_writer_[seg] = cur_;
+      for (int64_t r = g.rhead; r >= 0; r = rnext_[r]) dep(rtask_[r]);
+      g.rhead = -1;
+      g.writer = cur_;
     } else {
       grow4(rtask_);
       grow4(rnext_);
       rtask_.push_back(cur_);
-      rnext_.push_back(seg_rhead_[seg]);
-      seg_rhead_[seg] = (int64_t)rtask_.size() - 1;
+      rnext_.push_back(g.rhead);
+      g.rhead = (int64_t)rtask_.size() - 1;
     }
   }
   void acc(const MV& m, bool w) {
@@ -446,18 +457,26 @@ class Sched {
   }
   // Predecessors that another one already waits for order nothing more: they
   // are dropped when one of the kReduce latest predecessors lists them.  Every
-  // edge left costs its finishing task an atomic (n = 24: 94 M edges with all of them, 82 M without).
+  // edge left costs its finishing task an atomic (n = 24: 94 M edges with all of
+  // them, 82 M without).  Lists are ascending: only their end, from this task's
+  // first predecessor on, can name one of its predecessors.
   void end() {
     std::sort(deps_.begin(), deps_.end());
     if (deps_.size() > 1) {
       constexpr size_t kReduce = 8;
-      for (size_t k = 0; k < std::min(kReduce, deps_.size()); ++k) {
+      const int32_t first = deps_.front();
+      bool any = false;
+      for (size_t k = 0; k < std::min(kReduce, deps_.size() - 1); ++k) {
         const int32_t q = deps_[deps_.size() - 1 - k];
         if (implied_[q] == cur_) continue;
-        for (int64_t e = S_->pred_ptr[q]; e < S_->pred_ptr[q + 1]; ++e) implied_[S_->pred_idx[e]] = cur_;
+        for (int64_t e = S_->pred_ptr[q + 1] - 1; e >= S_->pred_ptr[q] && S_->pred_idx[e] >= first; --e) {
+          implied_[S_->pred_idx[e]] = cur_;
+          any = true;
+        }
       }
-      deps_.erase(std::remove_if(deps_.begin(), deps_.end(), [&](int32_t p) { return implied_[p] == cur_; }),
-                  deps_.end());
+      if (any)
+        deps_.erase(std::remove_if(deps_.begin(), deps_.end(), [&](int32_t p) { return implied_[p] == cur_; }),
+                    deps_.end());
     }
     grow4(S_->pred_idx, deps_.size());
     grow4(S_->pred_ptr);
@@ -515,12 +534,17 @@ class Sched {
   // only the few terms reading late_seg wait for the end of the preceding solve.
   void hmul(int32_t b, const MV& Vin, const MV& Vout, float sign, bool trans, bool overwrite, int32_t out_slot,
             int32_t late_seg = -1) {
-    std::vector<int32_t> lv;
+    // (scratch of this call, kept for its capacity)
+    std::vector<int32_t>&lv = hm_.leaves, &units = hm_.units, &cnt = hm_.cnt, &fill = hm_.fill, &items = hm_.items,
+        &part = hm_.part;
+    std::vector<MV>& T = hm_.T;
+    std::vector<int8_t>& group = hm_.group;
+    lv.clear();
     leaves_of(b, lv);
     int32_t oc = trans ? colc(b) : rowc(b);
     if (Vout.clus != oc || Vin.clus != (trans ? rowc(b) : colc(b)))
       throw std::logic_error("hmul cluster mismatch");
-    std::vector<MV> T(lv.size());
+    T.resize(lv.size());
     for (size_t i = 0; i < lv.size(); ++i) {
       int32_t be = lv[i];
       if (kind(be) != KIND_ADM) continue;
@@ -547,7 +571,7 @@ class Sched {
     }
     // output units: the segment clusters under the out-cluster (or the
     // out-cluster itself when it lies inside one segment)
-    std::vector<int32_t> units;
+    units.clear();
     if (seg_end_[oc] - seg_begin_[oc] <= 1) {
       units.push_back(oc);
     } else {
@@ -556,31 +580,37 @@ class Sched {
     const int32_t nu = (int32_t)units.size();
     const int32_t u0 = seg_begin_[oc];
     auto unit_of = [&](int32_t segidx) { return nu == 1 ? 0 : segidx - u0; };
-    std::vector<int32_t> cnt(nu + 1, 0);
+    cnt.assign(nu + 1, 0);
     for (size_t i = 0; i < lv.size(); ++i) {
       int32_t obc = trans ? colc(lv[i]) : rowc(lv[i]);
       for (int32_t q = seg_begin_[obc]; q < seg_end_[obc]; ++q) cnt[unit_of(q) + 1]++;
     }
     for (int32_t l = 0; l < nu; ++l) cnt[l + 1] += cnt[l];
-    std::vector<int32_t> fill(cnt.begin(), cnt.end() - 1), items(cnt[nu]);
+    fill.assign(cnt.begin(), cnt.end() - 1);
+    items.resize(cnt[nu]);
     for (size_t i = 0; i < lv.size(); ++i) {
       int32_t obc = trans ? colc(lv[i]) : rowc(lv[i]);
       for (int32_t q = seg_begin_[obc]; q < seg_end_[obc]; ++q) items[fill[unit_of(q)]++] = (int32_t)i;
     }
     MV kview = Vin;
+    group.resize(items.size());
     for (int32_t l = 0; l < nu; ++l) {
-      if (cnt[l] == cnt[l + 1] && !overwrite) continue;
-      constexpr int kGroups = 33;
-      std::vector<int32_t> parts[kGroups];
+      uint64_t used = overwrite ? 1 : 0;  // groups with a task
       for (int32_t q = cnt[l]; q < cnt[l + 1]; ++q) {
         int g = 0;
         if (late_seg >= 0 && !overwrite)
           for (int32_t dist = late_seg - (seg_end_[colc(lv[items[q]])] - 1); dist > 0; dist >>= 1) ++g;
-        parts[g].push_back(items[q]);
+        group[q] = (int8_t)g;
+        used |= uint64_t(1) << g;
       }
-      for (int part = kGroups - 1; part >= 0; --part)
-        if (!parts[part].empty() || (part == 0 && overwrite))
-          emit_rowmv(lv, T, parts[part], Vin, Vout, units[l], sign, trans, overwrite, out_slot, kview);
+      for (int g = 63; g >= 0 && used; --g) {
+        if (!(used >> g & 1)) continue;
+        used ^= uint64_t(1) << g;
+        part.clear();
+        for (int32_t q = cnt[l]; q < cnt[l + 1]; ++q)
+          if (group[q] == g) part.push_back(items[q]);
+        emit_rowmv(lv, T, part, Vin, Vout, units[l], sign, trans, overwrite, out_slot, kview);
+      }
     }
   }
   // the terms of a ROWMV task for unit lc, with their reads
@@ -672,8 +702,8 @@ class Sched {
     q.xoff = p.xoff;
     q.yoff = p.yoff;
     q.sign = p.sign;
-    q.pad = (alpha ? PF_ALPHA : 0) | (p.windows.empty() ? 0 : PF_DENSE);
-    for (int32_t b : p.windows) touch(bufs_[b].seg0, false);
+    q.pad = (alpha ? PF_ALPHA : 0) | (p.nwin == 0 ? 0 : PF_DENSE);
+    for (int32_t b = p.win0; b < p.win0 + p.nwin; ++b) touch(bufs_[b].seg0, false);
     grow4(S_->pieces);
     S_->pieces.push_back(q);
     acc(p.p.X, false);
@@ -735,7 +765,7 @@ class Sched {
         pending_fence_ = fences;
         const int32_t buf = new_buf_single();
         bind_alloc(buf);
-        out.windows.push_back(buf);
+        if (out.nwin++ == 0) out.win0 = buf;
         const int32_t wm = std::min(kWindow, m - wi), wn = std::min(kWindow, n - wj);
         std::vector<const PieceMV*> in;
         for (const PieceMV& p : ps)
@@ -1305,7 +1335,6 @@ class Sched {
   std::vector<int32_t>& dbuf_;
   std::vector<int32_t>& xbuf_;
   std::vector<int32_t>& ybuf_;
-  int32_t seg_size_of(int32_t) const { return segsz_; }
   int32_t segsz_ = 0;
   int64_t ring_off_ = 0, ring_size_ = 0, cursor_ = 0;
   bool accumulate_;
@@ -1323,24 +1352,21 @@ class Sched {
   int64_t forced_bucket_ = -kBuckets, update_seq_ = 0;
   std::vector<int32_t> pending_fence_;
   int64_t last_alloc_lo_ = 0, last_alloc_hi_ = -1, last_alloc_pos_ = 0;
-  int32_t fence_stamp_ = 0;
-  std::vector<int32_t> buf_fence_mark_;
-  std::vector<int64_t> fence_begin_, fence_end_;
   std::vector<int32_t> fence_pool_;
-  std::vector<int64_t> acc_head_;
-  std::vector<int32_t> acc_last_;
-  std::vector<int32_t> buf_chunk_, buf_pass_;  // a temporary's first chunk (else -1) and its pass
   std::vector<int32_t> acc_task_;
   std::vector<int64_t> acc_next_;
-  std::vector<int32_t> seg_buf_;
   std::vector<Buf> bufs_;
-  std::vector<int32_t> seg_writer_;
-  std::vector<int64_t> seg_rhead_;
+  std::vector<Seg> segs_;
   std::vector<int32_t> rtask_;
   std::vector<int64_t> rnext_;
   std::vector<int32_t> stamp_, implied_;
   std::vector<int32_t> deps_;
   int32_t cur_ = -1;
+  struct {
+    std::vector<int32_t> leaves, units, cnt, fill, items, part;
+    std::vector<MV> T;
+    std::vector<int8_t> group;
+  } hm_;                            // hmul's
   MV W_, Z_;                        // the solve's work vector and forward result
   std::vector<int32_t> blk_of_seg_, unit_of_seg_;  // solve block and diagonal tile of each segment
 };
@@ -1632,6 +1658,21 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bf
   const int32_t segsz = std::max(leafmax, tile);
   factor = Schedule();
   solve = Schedule();
+  // the solve's schedule is built beside the factorisation's, from a layout of
+  // its own (it adds nothing to it)
+  int64_t solve_temps = 0;
+  std::future<void> solved = std::async(std::launch::async | std::launch::deferred, [&, LS = L]() mutable {
+    // the solve's units are clusters of half a tile: a step of the chain spreads
+    // over twice as many SMs as with whole ones (n = 24, 8 columns: 8.4 -> 7.8 ms
+    // an apply, FP64 n = 11 5.2 -> 3.5 ms).  Smaller leaves are no units of their
+    // own: their edges are many (n = 16: 0.27 M with units of 32, 2.4 M with leaves
+    // of 8, 27 M with leaves of 2) and their rows leave lanes idle.
+    std::vector<int32_t> dbuf, xbuf, ybuf;
+    Sched s(C, B, rank_cap, LS, &solve, dbuf, xbuf, ybuf, true, std::max(leafmax, tile / 2), false, ring_off, ring);
+    s.solve_all(nrhs_max);
+    solve_temps = s.temp_elems_;
+    order_for_tickets(solve);
+  });
   std::vector<int32_t> dbuf, xbuf, ybuf;
   // accumulated updates hold factors for longer; where the ring is too small
   // for that, they are added at once
@@ -1644,17 +1685,8 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bf
     st.early_pieces = s.early_pieces_;
     st.accumulated = acc;
   });
-  {
-    // the solve's units are clusters of half a tile: a step of the chain spreads
-    // over twice as many SMs as with whole ones (n = 24, 8 columns: 8.4 -> 7.8 ms
-    // an apply, FP64 n = 11 5.2 -> 3.5 ms).  Smaller leaves are no units of their
-    // own: their edges are many (n = 16: 0.27 M with units of 32, 2.4 M with leaves
-    // of 8, 27 M with leaves of 2) and their rows leave lanes idle.
-    Sched s(C, B, rank_cap, L, &solve, dbuf, xbuf, ybuf, true, std::max(leafmax, tile / 2), false, ring_off, ring);
-    s.solve_all(nrhs_max);
-    st.temp_elems += s.temp_elems_;
-  }
-  order_for_tickets(solve);
+  solved.get();
+  st.temp_elems += solve_temps;
   factor.n_edges = (int64_t)factor.pred_idx.size();
   solve.n_edges = (int64_t)solve.pred_idx.size();
   st.n_factor_tasks = (int64_t)factor.tasks.size();
