@@ -57,11 +57,12 @@ def _factor_traffic(n, eps, precision, key="exec_kernel_factor", nrhs=None):
     """DRAM bytes per factorisation (key exec_kernel_factor) or preconditioner
     apply (exec_kernel_apply) launch recorded from an ncu capture in
     profiles/traffic.json, or None when that record is of another workload or
-    the executor source changed since it was taken."""
+    the executor's (or the solve's) source changed since it was taken."""
     try:
         with open(os.path.join(ROOT, "profiles", "traffic.json")) as f:
             rec = json.load(f)[key]
-        same_src = rec["exec_cu_blob"] == _blob_sha1(os.path.join(ROOT, "paper_2211_11303_gb300", "csrc", "exec.cu"))
+        same_src = all(rec[f + "_cu_blob"] == _blob_sha1(os.path.join(ROOT, "paper_2211_11303_gb300", "csrc", f + ".cu"))
+                       for f in ("exec", "solve") if f == "exec" or f + "_cu_blob" in rec)
         same_work = int(rec["n"]) == n and float(rec["eps"]) == eps and rec["precision"] == precision and (
             nrhs is None or int(rec.get("nrhs", -1)) == nrhs)
         return int(rec["dram_bytes_per_launch"]) if same_src and same_work else None
@@ -440,6 +441,7 @@ def run_gpu(args):
         try:
             hlu.hlu_factor(h, prec)
             info = hlu.hlu_factor_stats(h)
+            info["solve_bytes"] = hlu.hlu_solve_bytes(h)
             g0 = time.perf_counter()
             st = hlu.gmres_solve(h, Bd, X, restart=args.restart, tol=args.tol, maxit=args.maxit)
             st["gmres_ms"] = 1000.0 * (time.perf_counter() - g0)
@@ -503,7 +505,7 @@ def run_gpu(args):
     lat_sorted = sorted(lat)
     p99 = lat_sorted[min(len(lat_sorted) - 1, int(round(0.99 * (len(lat_sorted) - 1))))]
     apply_ms = statistics.mean(s["precond_ms"] / max(s["precond_applies"], 1) for s in sts)
-    live_bytes = statistics.mean(i["factor_live_bytes"] for i in infos)
+    live_bytes = statistics.mean(i["solve_bytes"] for i in infos)
     hbm_gbs = float(peaks.get("hbm_gbs", 6800.0))
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -542,11 +544,11 @@ def run_gpu(args):
                                "frac": live_bytes / (apply_ms / 1000.0) / 1e9 / hbm_gbs,
                                "traffic": _factor_traffic(n, args.eps, args.precision, "exec_kernel_apply", args.nrhs),
                                "bytes_per_apply": live_bytes,
-                               "kernel": "exec_kernel<float> (H-LU task executor), one triangular-solve "
-                                         "launch (L then U) per preconditioner apply",
+                               "kernel": "solve_kernel<float>, one triangular-solve launch (L then U) per "
+                                         "preconditioner apply",
                                "peak_source": "%s hbm_gbs" % src,
-                               "note": "algorithmic bytes = factor words at their live ranks, read once per "
-                                       "apply; time = CUDA events around the apply launches"}},
+                               "note": "algorithmic bytes = inverted diagonal blocks and the factor words at "
+                                       "their live ranks outside them, read once per apply; time = CUDA events around the apply launches"}},
         "clocks": clk,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": nrhs * N * 8,
                 "d2h_bytes_per_step": nrhs * N * 8},

@@ -129,7 +129,8 @@ typedef struct {
   int64_t factor_bytes;     /* device bytes of dense + low-rank factor storage   */
   int64_t workspace_bytes;  /* device bytes of temporaries and scratch           */
   double flops;             /* algorithmic flops of the factorisation (counted)  */
-  double factor_ms;         /* device time of the last hlu_factor                */
+  double factor_ms;         /* device time of the last hlu_factor, the inverses that
+                               the triangular solve multiplies with included      */
   double schedule_ms;       /* host time spent building the task DAG             */
   int32_t rank_max;         /* max rank of an admissible block after factoring   */
   int32_t rank_cap_hits;    /* truncations clipped at the rank capacity          */
@@ -139,8 +140,7 @@ typedef struct {
                                rank capacity + 1 when it asked for more          */
   int32_t trunc_dense_fallbacks; /* dense- or sampled-route truncations redone by the stack route */
   int64_t factor_live_bytes; /* bytes of the factor at its live ranks: dense words plus
-                                (rows + cols) x rank per admissible block; what one
-                                triangular-solve pass (L then U) reads            */
+                                (rows + cols) x rank per admissible block         */
   int32_t grid_ctas;        /* CTAs of the factorisation launch (persistent)       */
   int32_t reserved_;
 } hlu_factor_info;
@@ -407,6 +407,12 @@ int hlu_solve_batch(hlu_handle* const* hs, int32_t count, const double* const* b
  * handle at `precision` (factor storage + workspaces), for admission
  * control; -1 on error. */
 int64_t hlu_factor_bytes_estimate(const hlu_handle* h, int32_t precision);
+
+/* hlu_solve_bytes - factor bytes that one triangular solve (L then U) of a
+ * factored handle reads, each once: the row panels of the inverted diagonal
+ * blocks and, outside those blocks, dense words plus (rows + cols) x rank per
+ * admissible block.  -1 when the handle is not factored. */
+int64_t hlu_solve_bytes(const hlu_handle* h);
 
 /* hlu_set_wait_limit_ms - bound (milliseconds, default 20000) of every
  * device-side dependency wait; a wait that runs out sets HLU_ERR_TIMEOUT and

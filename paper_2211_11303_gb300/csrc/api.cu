@@ -317,6 +317,7 @@ struct hlu_handle {
   int32_t** d_rankp = nullptr;
   int32_t** d_pivp = nullptr;
   hlu_factor_info info;
+  int64_t solve_bytes = -1;  // hlu_solve_bytes
   KrylovWS kw;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   unsigned long long* d_prof = nullptr;  // executor profile of the last factorisation
@@ -1150,6 +1151,10 @@ int64_t hlu_factor_bytes_estimate(const hlu_handle* h, int32_t precision) {
   return h->L.total * es + grid * scratch_stride_elems(h->L, es) * es + (int64_t)h->L.n_slots * 4 + h->L.piv_total * 4;
 }
 
+int64_t hlu_solve_bytes(const hlu_handle* h) {
+  return h && h->precision >= 0 && !h->factor_pending ? h->solve_bytes : -1;
+}
+
 static int factor_impl(hlu_handle* h, int32_t precision, void* stream, int64_t limit);
 int hlu_factor(hlu_handle* h, int32_t precision, void* stream) {
   NvtxRange nvtx_("hlu_factor");
@@ -1257,6 +1262,13 @@ static int factor_finish(hlu_handle* h, hlu_handle* status_of, cudaStream_t s, f
   }
   const int es = esize(h->precision);
   h->info.factor_live_bytes = live * es;
+  // a solve multiplies with the inverses of the solve blocks in place of the
+  // leaves inside them
+  int64_t solve = live;
+  for (const InvLeaf& f : h->L.inv_leaves)
+    solve -= f.slot < 0 ? (int64_t)f.m * f.n : ((int64_t)f.m + f.n) * rk[f.slot];
+  for (const InvUnit& u : h->L.inv_units) solve += (int64_t)u.rows * (u.m + u.rows);
+  h->solve_bytes = solve * es;
   h->info.grid_ctas = h->grid;
   h->info.rank_max = rmax;
   h->info.rank_mean = nadm ? (double)rsum / nadm : 0.0;

@@ -103,6 +103,7 @@ SIGNATURES = {
     "hlu_set_preconditioner": (_i32, [_vp, _i32]),
     "hlu_solve_batch": (_i32, [_P(_vp), _i32, _P(_vp), _P(_vp), _P(_i32), _vp]),
     "hlu_factor_bytes_estimate": (_i64, [_vp, _i32]),
+    "hlu_solve_bytes": (_i64, [_vp]),
     "hlu_set_wait_limit_ms": (None, [_f64]),
     "hlu_set_tile": (None, [_i32]),
     "hlu_set_trunc_params": (_i32, [_i32, _f64]),
@@ -528,6 +529,11 @@ def hlu_solve_batch(handles, bs, xs, stream=None):
 
 def hlu_factor_bytes_estimate(h, precision=HLU_FP32):
     return int(lib().hlu_factor_bytes_estimate(_vp(h), int(precision)))
+
+
+def hlu_solve_bytes(h):
+    """Factor bytes that one triangular solve reads (-1: not factored)."""
+    return int(lib().hlu_solve_bytes(_vp(h)))
 
 
 def hlu_set_wait_limit_ms(ms):

@@ -104,3 +104,29 @@ def test_first_solve_of_a_factor_under_capture(hlu, prec):
     finally:
         hlu.hlu_destroy(h)
         hlu.hlu_destroy(other)
+
+
+def test_solve_bytes_count_what_a_solve_reads(hlu):
+    """One solve block (N <= 512): both triangles of its inverse and nothing of
+    the factor; more blocks: also the off-diagonal factor, less than the sum of
+    all panels and all live words."""
+    h = hlu.hlu_build(4, 2.0, 16, 2.0, 1e-4)
+    try:
+        assert hlu.hlu_solve_bytes(h) == -1
+        N = hlu.hlu_n(h)
+        assert N <= 512
+        for prec, es in ((hlu.HLU_FP32, 4), (hlu.HLU_FP64, 8)):
+            hlu.hlu_factor(h, prec)
+            # two triangles of units of at most 64 rows: N (N + rows of the unit) words
+            assert N * (N + 1) * es <= hlu.hlu_solve_bytes(h) <= N * (N + 64) * es
+    finally:
+        hlu.hlu_destroy(h)
+    h = hlu.hlu_build(8, 2.0, 16, 2.0, 1e-4)
+    try:
+        hlu.hlu_factor(h, hlu.HLU_FP32)
+        N = hlu.hlu_n(h)
+        live = hlu.hlu_factor_stats(h)["factor_live_bytes"]
+        panels = N * (512 + 64) * 4
+        assert N * 64 * 4 < hlu.hlu_solve_bytes(h) < live + panels
+    finally:
+        hlu.hlu_destroy(h)
