@@ -145,17 +145,17 @@ int hlu_debug_check_hazards(int32_t nc, const int32_t* clusters, int32_t nb, con
                             int32_t rank_cap, int32_t tile, int32_t nrhs_max, int32_t which, int64_t drop_edge,
                             int64_t* report);
 
-/* hlu_debug_check_hazards_ring - hlu_debug_check_hazards of the schedules that
- * the library uses at truncation tolerance eps, with a region for temporaries
- * of `ring` elements (0: the library's own size), so that a small mesh re-uses
- * its memory as often as a large one.  report: int64[15], the words above, then
+/* hlu_debug_check_hazards_ring - hlu_debug_check_hazards with the factorisation's
+ * updates accumulated (1), added at once (0) or as the library does at eps 1e-4
+ * (-1), and with a region for temporaries of `ring` elements (0: the library's
+ * own size), so that a small mesh re-uses its memory as often as a large one.  report: int64[15], the words above, then
  * of the factorisation (or Schulz step) the passes over the region beyond the
  * first, the updates added early to free their memory, whether updates were
  * accumulated (1 / 0), and the picked DAG's longest chain of truncations.  Returns as above; 6 also when the region cannot
  * hold the temporaries. */
 int hlu_debug_check_hazards_ring(int32_t nc, const int32_t* clusters, int32_t nb, const int32_t* blocks,
-                                 int32_t rank_cap, int32_t tile, int32_t nrhs_max, int32_t which, double eps,
-                                 int64_t ring, int64_t* report);
+                                 int32_t rank_cap, int32_t tile, int32_t nrhs_max, int32_t which,
+                                 int32_t accumulate, int64_t ring, int64_t* report);
 
 /* hlu_debug_host_hinverse - the Schulz inverse's task DAGs (hlu_hinverse)
  * run by the host reference executor in FP64 (no GPU): A_H from the CSR

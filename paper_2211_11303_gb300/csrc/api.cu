@@ -991,7 +991,7 @@ int hlu_build(const hlu_mesh* mesh, double kappa, int32_t leaf, double eta, doub
     uint64_t key = 1469598103934665603ULL;
     key = fnv1a(key, h->trees.clusters.data(), sizeof(int32_t) * h->trees.clusters.size());
     key = fnv1a(key, h->trees.blocks.data(), sizeof(int32_t) * h->trees.blocks.size());
-    const bool accumulate = accumulate_updates(h->tile, eps);
+    const bool accumulate = accumulate_updates((int32_t)N, h->tile, eps);
     int32_t params[5] = {rank_cap, h->tile, nrhs_max, (int32_t)N, accumulate ? 1 : 0};
     key = fnv1a(key, params, sizeof(params));
     bool cache_hit = false;

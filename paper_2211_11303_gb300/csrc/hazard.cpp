@@ -368,12 +368,13 @@ extern "C" int hlu_debug_check_hazards(int32_t nc, const int32_t* clusters, int3
 
 extern "C" int hlu_debug_check_hazards_ring(int32_t nc, const int32_t* clusters, int32_t nb, const int32_t* blocks,
                                             int32_t rank_cap, int32_t tile, int32_t nrhs_max, int32_t which,
-                                            double eps, int64_t ring, int64_t* report) {
-  if (ring < 0 || !report || !(eps > 0)) return 1;
+                                            int32_t accumulate, int64_t ring, int64_t* report) {
+  if (ring < 0 || !report || !clusters || nc < 1 || accumulate < -1 || accumulate > 1) return 1;
   SchedStats st;
   report[11] = report[12] = report[13] = report[14] = 0;
   const int rc = check_hazards(nc, clusters, nb, blocks, rank_cap, tile, nrhs_max, which, -1,
-                               accumulate_updates(tile, eps), ring, report, st, report + 14);
+                               accumulate < 0 ? accumulate_updates(clusters[1], tile, 1e-4) : accumulate != 0, ring,
+                               report, st, report + 14);
   if (rc == 0 || rc == 9) {
     report[11] = st.ring_wraps;
     report[12] = st.early_pieces;

@@ -166,7 +166,7 @@ void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& B,
                      Schedule& factor, Schedule& solve, SchedStats& st, std::vector<Block>* factor_blocks,
                      bool accumulate, int64_t ring_elems = 0);
 // Whether the library accumulates the updates of a factorisation.
-bool accumulate_updates(int32_t tile, double eps);
+bool accumulate_updates(int32_t N, int32_t tile, double eps);
 std::vector<Block> factor_tree(const std::vector<Cluster>& C, const std::vector<Block>& B, int32_t tile);
 
 // The Schulz iteration for the inverse of A_H (Sec. 3, Sec. 4) over four

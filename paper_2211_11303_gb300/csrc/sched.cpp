@@ -1578,13 +1578,19 @@ void with_ring(bool accumulate, ArenaLayout& L, const F& build) {
 // Without tiles (tile 0: the block tree's own small leaves) the accumulated
 // updates of a leaf are many and make one long chain of truncations: n = 10,
 // leaf 16: 517 ms against 63 ms added at once (FP64, n = 8: 1,838 against 118
-// ms).  With tiles the two take about the same time at eps 1e-3 to 1e-5 (n =
-// 24, FP32, eps 1e-4: 713 against 710 ms), and the accumulated factor is the
-// nearer one (one apply leaves 2e-3 of the residual against 1e-2, n = 24).  At
-// finer eps the sums' spectra are filled with rounding and the wide truncations
-// cost more: n = 16, FP32: 1e-6 374 against 267 ms, 1e-7 697 against 453 ms; n =
-// 11, FP64, 1e-10: 529 against 474 ms.
-bool accumulate_updates(int32_t tile, double eps) { return tile > 0 && eps >= 4e-6; }
+// ms).  With tiles the two take about the same time at coarse eps (n = 24, FP32,
+// eps 1e-4: 713 against 710 ms), and the accumulated factor is the nearer one
+// (one apply leaves 2e-3 of the residual against 1e-2, n = 24).  At finer eps the
+// sums' spectra are filled with rounding and the wide truncations cost more, the
+// more the larger the mesh.  FP32, accumulated against at once: eps 1e-5 n = 13
+// 70.8 : 71.6 (with the solve), n = 16 172 : 155, n = 24 1,126 : 901 ms, at
+// kappa 16 n = 24 1.62 : 1.07, n = 32 5.83 : 3.53, n = 40 21.0 : 12.3 s; eps 1e-6
+// n = 16 374 : 268, n = 24 2,600 : 1,496 ms.  FP64: eps 1e-6 n = 8 65 : 73, n =
+// 11 316 : 311 ms; 1e-12 n = 8 73 : 88, n = 11 576 : 521 ms.  (n = 8: N = 3,032;
+// 11: 8,261; 13: 13,897; 16: 26,416.)
+bool accumulate_updates(int32_t N, int32_t tile, double eps) {
+  return tile > 0 && (eps >= 3e-5 || N < 5000 || (eps >= 4e-6 && N < 20000));
+}
 
 void build_schedules(const std::vector<Cluster>& C, const std::vector<Block>& Bfull, int32_t rank_cap,
                      int32_t nrhs_max, int32_t tile, ArenaLayout& L,
